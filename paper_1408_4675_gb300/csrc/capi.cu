@@ -243,6 +243,7 @@ extern "C" int kwgb_create(const kwgb_grid_desc* desc, kwgb_sim** out) {
     g.nx = (int)n[0]; g.ny = (int)n[1]; g.nz = (int)n[2];
     g.nh = g.nx / 2 + 1;
     g.nhp = (g.nh + 15) / 16 * 16;
+    g.lb = spec_block_log2(g.nx);
     g.lognx = ilog2(n[0]); g.logny = ilog2(n[1]); g.lognz = ilog2(n[2]);
     g.dt = (float)desc->dt;
     sim->N = n[0] * n[1] * n[2];
@@ -257,7 +258,7 @@ extern "C" int kwgb_create(const kwgb_grid_desc* desc, kwgb_sim** out) {
     g.abs_e[1] = (float)((y - 1.0) / 2.0);
     g.abs_c[0] = (float)std::pow(std::sqrt(kmax2), y - 2.0);
     g.abs_c[1] = (float)std::pow(std::sqrt(kmax2), y - 1.0);
-    sim->spec_elems = (size_t)g.nhp * g.ny * g.nz;
+    sim->spec_elems = spec_elems(g);
     Medium& md = sim->md;
     std::memset(&md, 0, sizeof(md));
     md.y = (float)y;
@@ -422,7 +423,7 @@ extern "C" int kwgb_set_medium(kwgb_sim* sim, const float* c0, const float* rho0
     DALLOC(sim->T1, float2, sim->spec_elems);
     DALLOC(sim->T2, float2, sim->spec_elems);
     DALLOC(sim->T3, float2, sim->spec_elems);
-    CK(cudaMemset(sim->P, 0, sim->spec_elems * sizeof(float2)));
+    for (float2* p : {sim->P, sim->T1, sim->T2, sim->T3}) CK(cudaMemset(p, 0, sim->spec_elems * sizeof(float2)));
     {
         int sms = 0;
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id));
@@ -983,7 +984,7 @@ static std::vector<std::pair<void*, size_t>> state_blocks(kwgb_sim* sim) {
     const size_t F = (size_t)sim->N * sizeof(float);
     for (int a = 0; a < 3; ++a) b.push_back({sim->u[a], F});
     for (int a = 0; a < 3; ++a) b.push_back({sim->rho[a], F});
-    b.push_back({sim->P, sim->spec_elems * sizeof(float2)});
+    b.push_back({sim->P, (size_t)sim->g.nhp * sim->g.ny * sim->g.nz * sizeof(float2)});   // (as whole rows)
     const SensorC& sc = sim->sens;
     if (sim->n_slots) {
         b.push_back({sc.p_max, sim->n_slots * sizeof(float)});
@@ -1035,8 +1036,9 @@ extern "C" int kwgb_save_state(kwgb_sim* sim, void* buf, int64_t len) {
     char* out = static_cast<char*>(buf);
     std::memcpy(out, &h, sizeof(h));
     size_t off = sizeof(h);
+    CK(launch_spec_rows(sim->g, sim->P, sim->T3, true, nullptr));   // a snapshot holds P as whole rows
     for (auto& b : state_blocks(sim)) {
-        CK(cudaMemcpy(out + off, b.first, b.second, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(out + off, b.first == sim->P ? sim->T3 : b.first, b.second, cudaMemcpyDeviceToHost));
         off += b.second;
     }
     return KWGB_OK;
@@ -1059,9 +1061,11 @@ extern "C" int kwgb_load_state(kwgb_sim* sim, const void* buf, int64_t len) {
     const char* in = static_cast<const char*>(buf);
     size_t off = sizeof(h);
     for (auto& b : state_blocks(sim)) {
-        CK(cudaMemcpy(b.first, in + off, b.second, cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(b.first == sim->P ? sim->T3 : b.first, in + off, b.second, cudaMemcpyHostToDevice));
         off += b.second;
     }
+    CK(launch_spec_rows(sim->g, sim->T3, sim->P, false, nullptr));
+    CK(cudaDeviceSynchronize());
     CK(cudaMemcpy(sim->d_step, &h.steps, sizeof(int64_t), cudaMemcpyHostToDevice));
     CK(cudaMemset(sim->d_flag, 0, sizeof(int)));
     sim->steps = h.steps;
@@ -1203,7 +1207,7 @@ extern "C" int kwgb_read(kwgb_sim* sim, int32_t sensor_id, uint32_t which, doubl
         LK(launch_intensity_gather(sim->n_i, sim->i_idx, g, sim->u, g.nx, sim->ubuf, s));
         float* tails[3] = {reinterpret_cast<float*>(out[0]), reinterpret_cast<float*>(out[1]),
                            reinterpret_cast<float*>(out[2])};
-        LK(launch_intensity_accum(sim->n_i, sim->i_idx, g, tails, 2 * g.nhp, sim->ubuf, sc.p_sens,
+        LK(launch_intensity_accum(sim->n_i, sim->i_idx, g, tails, 0, sim->ubuf, sc.p_sens,
                                   sim->i_slot, sim->I_tail, sim->d_step, 0, s));
         CK(cudaDeviceSynchronize());
         std::vector<double> a(3 * sim->n_i), b(3 * sim->n_i);

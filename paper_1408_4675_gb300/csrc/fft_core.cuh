@@ -40,6 +40,19 @@ __host__ __device__ constexpr float cos16(int m) {
          : -1.0f;
 }
 __host__ __device__ constexpr float sin16(int m) { return cos16(m - 4); }
+// cos and sin(2 pi m / 32)
+__host__ __device__ constexpr float cos32(int m) {
+    return (m & 1) == 0 ? cos16(m >> 1)
+         : (m & 31) == 1 || (m & 31) == 31 ? 0.98078528040323044913f
+         : (m & 31) == 3 || (m & 31) == 29 ? 0.83146961230254523708f
+         : (m & 31) == 5 || (m & 31) == 27 ? 0.55557023301960222474f
+         : (m & 31) == 7 || (m & 31) == 25 ? 0.19509032201612826785f
+         : (m & 31) == 9 || (m & 31) == 23 ? -0.19509032201612826785f
+         : (m & 31) == 11 || (m & 31) == 21 ? -0.55557023301960222474f
+         : (m & 31) == 13 || (m & 31) == 19 ? -0.83146961230254523708f
+         : -0.98078528040323044913f;
+}
+__host__ __device__ constexpr float sin32(int m) { return cos32(m - 8); }
 
 // d * exp(DIR * 2 pi i * m / 16) for a compile-time m (after unrolling).
 template <int DIR>
@@ -93,8 +106,8 @@ __device__ __forceinline__ void dft_reg(float2* v) {
     }
 }
 
-// The twiddle table (Tables::tw, float2, generated in float64) has three
-// regions; every entry is exp(-2 pi i theta):
+// The twiddle table (Tables::tw, float2, generated in float64) has four
+// regions; every entry of the first three is exp(-2 pi i theta):
 //   [0, 1024)            theta = t / 1024
 //   stage blocks         one per (L, RP), at stw_off(L, RP): entry (r-1) L/RP + k
 //                        holds theta = k r / L for k < L/RP, 1 <= r < RP -- the
@@ -114,7 +127,18 @@ __host__ __device__ constexpr int stw_off(int L, int RP) {
     return off;
 }
 __host__ __device__ constexpr int rtw_off(int M) { return stw_off(2048, 2) + M - 2; }
-constexpr int TW_TOTAL = rtw_off(1024);            // entries of the whole table
+constexpr int TW_SINGLE = (rtw_off(1024) + 1) / 2 * 2;   // entries of the regions above
+// A fourth region serves the lines of 32 values per thread (line_pass.cuh),
+// three blocks (N = 256, 512, 1024) at twh_off(log2 N), TL = N / 32:
+//   u < 16, j < TL: float4 (c, c', s, s') at index u TL + j, theta = 2 u j / N in
+//                   (c, s) and (2 u + 1) j / N in (c', s')
+//   N < 1024: r < TL, b < 16: the same at index 16 TL + 16 r + b, theta = 2 b r / N and
+//                   (2 b + 1) r / N
+//   N = 1024: r < 32, j < 32: float2 at float2 index 32 TL + 32 r + j, theta = j r / N
+__host__ __device__ constexpr int twh_off(int logn) {
+    return TW_SINGLE + (logn > 8 ? 2 * (16 * 8 + 8 * 16) : 0) + (logn > 9 ? 2 * (16 * 16 + 16 * 16) : 0);
+}
+constexpr int TW_TOTAL = twh_off(10) + 2 * 16 * 32 + 32 * 32;   // entries of the whole table
 
 // exp(DIR 2 pi i k r / L) of a radix-RP pass building length-L transforms.
 template <int DIR, int L, int RP>

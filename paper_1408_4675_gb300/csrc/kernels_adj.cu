@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_absprep_ke
         q1[m] = make_float2(ct.x * l.x, ct.y * l.y);
         q2[m] = make_float2(ct.x * c.x * md.tan_pi_y_2 * l.x, ct.y * c.y * md.tan_pi_y_2 * l.y);
     }
-    row_r2c<LOGM>(q1, S, j, valid, g.t.tw, K.a.sp[0] + (size_t)rr * g.nhp);
-    row_r2c<LOGM>(q2, S, j, valid, g.t.tw, K.a.sp[1] + (size_t)rr * g.nhp);
+    row_r2c<LOGM>(q1, S, j, valid, g.t.tw, spec_row<Sh::M>(K.a.sp[0], rr), g);
+    row_r2c<LOGM>(q2, S, j, valid, g.t.tw, spec_row<Sh::M>(K.a.sp[1], rr), g);
 }
 
 template <int LOGM, bool ABS>
@@ -113,10 +113,10 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_dens_kerne
     }
     if (ABS) {                                        // Eq. 8 backwards: a1 -> lambda_d, a2 -> lambda_rho
         float2 a[E];
-        row_c2r<LOGM>(K.a.sp[0] + (size_t)rr * g.nhp, S, j, valid, g.t.tw, a);
+        row_c2r<LOGM>(spec_row<Sh::M>(K.a.sp[0], rr), g, S, j, valid, g.t.tw, a);
 #pragma unroll
         for (int m = 0; m < E; ++m) labs[m] = make_float2(r0[m].x * a[m].x, r0[m].y * a[m].y);
-        row_c2r<LOGM>(K.a.sp[1] + (size_t)rr * g.nhp, S, j, valid, g.t.tw, a);
+        row_c2r<LOGM>(spec_row<Sh::M>(K.a.sp[1], rr), g, S, j, valid, g.t.tw, a);
 #pragma unroll
         for (int m = 0; m < E; ++m) lrt[m] = cadd(lrt[m], a[m]);
     }
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_dens_kerne
             if (valid) st2(pick3f(K.a.lam_rho, xi) + i, nlr);
             v[m] = ld;
         }
-        row_r2c<LOGM>(v, S, j, valid, g.t.tw, pick3w(K.a.sp, xi) + (size_t)rr * g.nhp);
+        row_r2c<LOGM>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(pick3w(K.a.sp, xi), rr), g);
     }
     if (valid) {
 #pragma unroll
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_vel_kernel
             else r1[m] = ldg2(rho0 + nb + x);
         }
         float2 v[E];
-        row_c2r<LOGM>(pick3w(K.a.sp, xi) + (size_t)rr * g.nhp, S, j, valid, g.t.tw, v);
+        row_c2r<LOGM>(spec_row<Sh::M>(pick3w(K.a.sp, xi), rr), g, S, j, valid, g.t.tw, v);
         const float fyz = xi == 1 ? __ldg(g.t.pml_sg[1] + y) : __ldg(g.t.pml_sg[2] + z);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_vel_kernel
             if (valid) st2(lu + rb + x, make_float2(f.x * f.x * lup.x, f.y * f.y * lup.y));
             v[m] = make_float2(-__fdividef(f.x * g.dt * lup.x, rs.x), -__fdividef(f.y * g.dt * lup.y, rs.y));
         }
-        row_r2c<LOGM>(v, S, j, valid, g.t.tw, pick3w(K.a.sp, xi) + (size_t)rr * g.nhp);
+        row_r2c<LOGM>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(pick3w(K.a.sp, xi), rr), g);
     }
 }
 
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_p_kernel(c
     const int rr = valid ? row : 0;
     typename Sh::Smem S = Sh::row_smem(smem, r);
     float2 v[E];
-    row_c2r<LOGM>(K.a.sp[0] + (size_t)rr * g.nhp, S, j, valid, g.t.tw, v);
+    row_c2r<LOGM>(spec_row<Sh::M>(K.a.sp[0], rr), g, S, j, valid, g.t.tw, v);
     if (valid) {
 #pragma unroll
         for (int m = 0; m < E; ++m)

@@ -23,6 +23,23 @@ void fill_twiddle_table(float2* out) {
         }
     for (int M = 2; M <= 512; M *= 2)
         for (int k = 0; k < M; ++k) out[rtw_off(M) + k] = unit_root(k, 2 * M);
+    auto pair = [&](float2* o, long a, long b, long n) {
+        const float2 w = unit_root(a, n), v = unit_root(b, n);
+        o[0] = make_float2(w.x, v.x);
+        o[1] = make_float2(w.y, v.y);
+    };
+    for (int logn = 8; logn <= 10; ++logn) {
+        const long n = 1 << logn, tl = n / 32;
+        float2* o = out + twh_off(logn);
+        for (long u = 0; u < 16; ++u)
+            for (long j = 0; j < tl; ++j) pair(o + 2 * (u * tl + j), 2 * u * j, (2 * u + 1) * j, n);
+        for (long r = 0; r < tl; ++r) {
+            if (logn < 10)
+                for (long b = 0; b < 16; ++b) pair(o + 32 * tl + 2 * (16 * r + b), 2 * b * r, (2 * b + 1) * r, n);
+            else
+                for (long j = 0; j < 32; ++j) o[32 * tl + 32 * r + j] = unit_root(j * r, n);
+        }
+    }
 }
 
 __global__ void init_rho_kernel(GridC g, Medium md, const float* __restrict__ p0, int pitch,
@@ -91,6 +108,22 @@ cudaError_t launch_advance_step(int64_t* step, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+__global__ void spec_rows_kernel(GridC g, const float2* __restrict__ in, float2* __restrict__ out, bool to_rows) {
+    const int64_t n = (int64_t)g.nhp * g.ny * g.nz;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t row = i / g.nhp;
+        const int col = (int)(i % g.nhp);
+        const size_t b = spec_off(g, col, (int)(row % g.ny), (int)(row / g.ny));
+        if (to_rows) out[i] = in[b];
+        else out[b] = in[i];
+    }
+}
+
+cudaError_t launch_spec_rows(const GridC& g, const float2* in, float2* out, bool to_rows, cudaStream_t s) {
+    spec_rows_kernel<<<1216, 256, 0, s>>>(g, in, out, to_rows);
+    return cudaGetLastError();
+}
+
 __global__ void fill_f32_kernel(float* p, int64_t n, float v) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -114,8 +147,12 @@ __device__ __forceinline__ void neighbours(int64_t s, const GridC& g, int64_t (&
     nb[2] = x + g.nx * (y + (int64_t)g.ny * ((z + g.nz - 1) % g.nz));
 }
 
+// float index of grid point i in rows of `pitch` floats, or (pitch 0) in the real rows of a spectrum buffer
 __device__ __forceinline__ int64_t pitched(int64_t i, const GridC& g, int pitch) {
-    return (i / g.nx) * pitch + (i % g.nx);
+    const int64_t row = i / g.nx, x = i % g.nx;
+    if (pitch > 0) return row * pitch + x;
+    const int64_t n = x >> 1;
+    return 2 * ((n >> g.lb) * (int64_t)spec_block(g) + (row << g.lb) + (n & ((1 << g.lb) - 1))) + (x & 1);
 }
 
 struct UPtrs {

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_dens_kernel(co
     const size_t NN = (size_t)g.nx * g.ny * g.nz;
     float* kp = nullptr;                               // this step's kept fields
     if (DOUT) kp = K.a.keep + (size_t)(*K.st.step % K.a.keep_period) * 7 * NN;
-    if (mygroups > 0) stage_rows<LOGM>(stage, K.a.D[0], gw * RPW, nrows, g.nhp, lane);
+    if (mygroups > 0) stage_rows<LOGM>(stage, K.a.D[0], gw * RPW, nrows, g, lane);
     cp_async_commit();
     for (int gi = 0; gi < mygroups; ++gi) {
         const int grp = gw + gi * nw;
@@ -66,10 +66,10 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_dens_kernel(co
             const int it = 3 * gi + xi;
             S.sync();
             if (xi < 2) stage_rows<LOGM>(stage + ((it + 1) & 1) * RPW * St::SROW, pick3(K.a.D, xi + 1), grp * RPW,
-                                         nrows, g.nhp, lane);
+                                         nrows, g, lane);
             else if (gi + 1 < mygroups)
                 stage_rows<LOGM>(stage + ((it + 1) & 1) * RPW * St::SROW, K.a.D[0], (grp + nw) * RPW, nrows,
-                                 g.nhp, lane);
+                                 g, lane);
             cp_async_commit();
             float* rho_xi = pick3f(K.a.rho, xi);
             float2 ro_[E], r0[E];                     // issued before the row transform (rho0: L1/L2 hits)
@@ -199,10 +199,10 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_dens_kernel(co
             if (valid) {
 #pragma unroll
                 for (int m = 0; m < E; ++m)
-                    st2(K.a.rho_tot + (size_t)rr * 2 * g.nhp + 2 * (j + TL * m), rt[m]);
+                    __stcs(spec_at<Sh::M>(spec_row<Sh::M>(reinterpret_cast<float2*>(K.a.rho_tot), rr), g, j + TL * m), rt[m]);
             }
-            row_r2c<LOGM>(s, S, j, valid, g.t.tw, K.a.S + (size_t)rr * g.nhp);
-            row_r2c<LOGM>(rt, S, j, valid, g.t.tw, K.a.R + (size_t)rr * g.nhp);
+            row_r2c<LOGM>(s, S, j, valid, g.t.tw, spec_row<Sh::M>(K.a.S, rr), g);
+            row_r2c<LOGM>(rt, S, j, valid, g.t.tw, spec_row<Sh::M>(K.a.R, rr), g);
         }
     }
 }
@@ -218,9 +218,10 @@ struct XEosK {
 };
 
 // Copy rows first_row .. first_row + RPT - 1 of a real field (nx = 2M floats
-// per row, row pitch `pitch` floats) into dst (M float2 per row).
+// per row, `pitch` floats between rows, `step` floats between a row's pieces
+// of 2^lb float2) into dst (M float2 per row).
 template <int LOGM>
-__device__ __forceinline__ void stage_real_rows(float2* dst, const float* __restrict__ src, size_t pitch,
+__device__ __forceinline__ void stage_real_rows(float2* dst, const float* __restrict__ src, size_t pitch, size_t step, int lb,
                                                 int first_row, int nrows, int lane) {
     using Sh = XShape<LOGM>;
     constexpr int CH = Sh::M / 2;                        // 16-byte chunks per row
@@ -229,7 +230,7 @@ __device__ __forceinline__ void stage_real_rows(float2* dst, const float* __rest
         const int c = lane + Sh::TEAM * t;
         if (c < Sh::RPT * CH) {
             const int r = c / CH, q = c % CH;
-            if (first_row + r < nrows) cp_async16(dst + r * Sh::M + 2 * q, src + (size_t)(first_row + r) * pitch + 4 * q);
+            if (first_row + r < nrows) cp_async16(dst + r * Sh::M + 2 * q, src + (size_t)(first_row + r) * pitch + ((2 * q) >> lb) * step + 2 * ((2 * q) & ((1 << lb) - 1)));
         }
     }
 }
@@ -265,11 +266,12 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_eos_kernel(con
     float2* stage = smem + Sh::RPB * Sh::PITCH + team * Es::TEAM;
     const int first = blockIdx.x * Sh::RPB + team * Sh::RPT;
     const bool nl = md.nonlinear;
-    stage_rows<LOGM>(stage, K.a.A1, first, nrows, g.nhp, lane);
-    stage_rows<LOGM>(stage + Es::A, K.a.A2, first, nrows, g.nhp, lane);
-    stage_real_rows<LOGM>(stage + 2 * Es::A, K.a.rho_tot, 2 * (size_t)g.nhp, first, nrows, lane);
-    if (nl && md.rho0) stage_real_rows<LOGM>(stage + 2 * Es::A + Es::R, md.rho0, g.nx, first, nrows, lane);
-    if (nl && md.bona) stage_real_rows<LOGM>(stage + 2 * Es::A + 2 * Es::R, md.bona, g.nx, first, nrows, lane);
+    stage_rows<LOGM>(stage, K.a.A1, first, nrows, g, lane);
+    stage_rows<LOGM>(stage + Es::A, K.a.A2, first, nrows, g, lane);
+    // rho: real rows of a spectrum buffer; the medium's rows: one piece each
+    stage_real_rows<LOGM>(stage + 2 * Es::A, K.a.rho_tot, (size_t)2 << spec_block_log2(2 * M), 2 * spec_block(g), spec_block_log2(2 * M), first, nrows, lane);
+    if (nl && md.rho0) stage_real_rows<LOGM>(stage + 2 * Es::A + Es::R, md.rho0, g.nx, 0, 30, first, nrows, lane);
+    if (nl && md.bona) stage_real_rows<LOGM>(stage + 2 * Es::A + 2 * Es::R, md.bona, g.nx, 0, 30, first, nrows, lane);
     cp_async_commit();
     const size_t rb = (size_t)rr * g.nx;
     const int lr = r % Sh::RPT;                          // this row within the team's stage
@@ -357,7 +359,7 @@ __global__ void __launch_bounds__(XTHREADS) x_r2c_kernel(const XPlainK K) {
 #pragma unroll
     for (int m = 0; m < E; ++m)
         v[m] = valid ? ld2(K.rin + (size_t)rr * K.rpitch + 2 * (j + TL * m)) : make_float2(0.f, 0.f);
-    row_r2c<LOGM>(v, S, j, valid, K.g.t.tw, K.cout + (size_t)rr * K.g.nhp);
+    row_r2c<LOGM>(v, S, j, valid, K.g.t.tw, spec_row<Sh::M>(K.cout, rr), K.g);
 }
 
 template <int LOGM>
@@ -371,7 +373,7 @@ __global__ void __launch_bounds__(XTHREADS) x_c2r_kernel(const XPlainK K) {
     const int rr = valid ? row : 0;
     typename Sh::Smem S = Sh::row_smem(smem, r);
     float2 v[E];
-    row_c2r<LOGM>(K.cin + (size_t)rr * K.g.nhp, S, j, valid, K.g.t.tw, v);
+    row_c2r<LOGM>(spec_row<Sh::M>(K.cin, rr), K.g, S, j, valid, K.g.t.tw, v);
     if (valid) {
 #pragma unroll
         for (int m = 0; m < E; ++m) st2(K.rout + (size_t)rr * K.rpitch + 2 * (j + TL * m), v[m]);

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(con
             else r1[m] = ldg2(rho0 + nb + x);
         }
         float2 v[E];
-        row_c2r<LOGM>(K.a.G[xi] + (size_t)rr * g.nhp, S, j, valid, g.t.tw, v);
+        row_c2r<LOGM>(spec_row<Sh::M>(K.a.G[xi], rr), g, S, j, valid, g.t.tw, v);
         const float fyz = xi == 1 ? __ldg(g.t.pml_sg[1] + y) : __ldg(g.t.pml_sg[2] + z);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(con
                                  f.y * (f.y * uo[m].y - __fdividef(g.dt * gr.y, rs.y)));
             }
             if (valid) {
-                if (MODE == XV_TAIL) st2(K.a.tail[xi] + (size_t)rr * 2 * g.nhp + x, un);
+                if (MODE == XV_TAIL) __stcs(spec_at<Sh::M>(spec_row<Sh::M>(reinterpret_cast<float2*>(K.a.tail[xi]), rr), g, x >> 1), un);
                 else st2(K.a.u[xi] + rb + x, un);
             }
             v[m] = un;
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(con
                     }
                     const float un = S.f(x) + __fdividef(acc, rsx);
                     S.f(x) = un;
-                    if (MODE == XV_TAIL) K.a.tail[xi][(size_t)rr * 2 * g.nhp + x] = un;
+                    if (MODE == XV_TAIL) reinterpret_cast<float*>(spec_at<Sh::M>(spec_row<Sh::M>(reinterpret_cast<float2*>(K.a.tail[xi]), rr), g, x >> 1))[x & 1] = un;
                     else K.a.u[xi][rb + x] = un;
                 }
             }
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(con
                 }
             }
         }
-        if (MODE == XV_STEP) row_r2c<LOGM>(v, S, j, valid, g.t.tw, K.a.U[xi] + (size_t)rr * g.nhp);
+        if (MODE == XV_STEP) row_r2c<LOGM>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(K.a.U[xi], rr), g);
     }
 }
 

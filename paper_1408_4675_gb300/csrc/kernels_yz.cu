@@ -29,11 +29,14 @@ static int encode_box(const GridC& g, float2* ptr, CUtensorMap* map) {
     using Sh = TShape<LOGN, ISY, MIXED>;
     EncodeTiledFn fn = encode_fn();
     if (!fn) return -1;
-    const cuuint64_t dims[3] = {(cuuint64_t)g.nh, (cuuint64_t)g.ny, (cuuint64_t)g.nz};
-    const cuuint64_t strides[2] = {(cuuint64_t)g.nhp * 8, (cuuint64_t)g.ny * g.nhp * 8};
-    const cuuint32_t box[3] = {(cuuint32_t)Sh::CX, ISY ? (cuuint32_t)Sh::BOX : 1u, ISY ? 1u : (cuuint32_t)Sh::BOX};
-    const cuuint32_t es[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 3, ptr, dims, strides, box, es,
+    // 16-column blocks: a tile's CX columns lie in one block (CX divides 16)
+    static_assert(16 % Sh::CX == 0, "tile width");
+    const cuuint64_t w = (cuuint64_t)1 << g.lb, row = w * 8;
+    const cuuint64_t dims[4] = {w, (cuuint64_t)g.ny, (cuuint64_t)g.nz, (g.nh + w - 1) / w};
+    const cuuint64_t strides[3] = {row, g.ny * row, (cuuint64_t)g.ny * g.nz * row};
+    const cuuint32_t box[4] = {(cuuint32_t)Sh::CX, ISY ? (cuuint32_t)Sh::BOX : 1u, ISY ? 1u : (cuuint32_t)Sh::BOX, 1u};
+    const cuuint32_t es[4] = {1, 1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 4, ptr, dims, strides, box, es,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? 0 : -2;
@@ -99,6 +102,7 @@ cudaError_t launch_z_op(const GridC& g, int kind, const SpecBuf* const* in, floa
     a.g = g;
     a.flag = flag;
     for (int i = 0; i < 3; ++i) a.out[i] = out[i];
+    a.short_kappa = g.hk2 <= 1.9999f * g.inv_kmax2;   // with room for the rounding of k^2
     if (kind == Z_GRAD_FWD || kind == Z_GRAD_BWD) {
         a.map[0] = in[0]->zmap;
         a.nloads = 1;

@@ -33,7 +33,8 @@ struct Tables {
 struct GridC {
     int nx, ny, nz;           // grid
     int nh;                   // nx / 2 + 1 (half-spectrum length along x)
-    int nhp;                  // row pitch of spectra, complex elements (multiple of 16)
+    int nhp;                  // nh rounded up to a multiple of 16 (row pitch of a snapshot)
+    int lb;                   // log2 of the columns of a spectrum block (spec_off)
     int lognx, logny, lognz;
     float dt;
     float scale;              // 1 / (nx ny nz): inverse-FFT normalisation
@@ -47,6 +48,25 @@ struct GridC {
     uint32_t wait_fault_tx;   // test hook (kwgb_debug_wait_fault): extra bytes each tile load expects, 0 normally
     Tables t;
 };
+
+// Layout of a spectrum: blocks of 2^lb columns, [blocks][nz][ny][2^lb] complex,
+// 32 columns (256-byte pieces of a row) for rows longer than 64 reals, else 16.
+// A line along y strides one piece, a line along z ny pieces.  With whole rows
+// ([nz][ny][nx/2 + 1]) the stride along z is 4.3 MB at 1024^3, so that every
+// element of a z line lies in a 2 MB page of its own and the z passes are bound by
+// address translation: z_abs 2.8 TB/s at 1024^3, against 4.4 TB/s on the same lines
+// with a 0.28 MB stride.  Measured step times over the block width at 512^3 / 1024^3:
+// 16 columns 8.15 / 67.4 ms, 32 7.90 / 67.0, 64 7.91 / 67.4, 128 7.95 / 69.0, one block
+// of 512 or 1024 (a power-of-two stride) 8.53 / 75.4, whole rows 8.00 / 73.7: wide pieces serve
+// the x passes, short strides the z passes.
+// Real rows of nx values kept in a spectrum buffer (rho_tot, tail) take the row's own
+// place in it: the float2 (x = 2n, 2n + 1) is complex element n.
+__host__ __device__ constexpr int spec_block_log2(int nx) { return nx > 64 ? 5 : 4; }
+__host__ __device__ inline size_t spec_block(const GridC& g) { return ((size_t)g.ny * g.nz) << g.lb; }   // elements per block
+__host__ __device__ inline size_t spec_off(const GridC& g, int col, int y, int z) {
+    return (size_t)(col >> g.lb) * spec_block(g) + (((size_t)z * g.ny + y) << g.lb) + (col & ((1 << g.lb) - 1));
+}
+inline size_t spec_elems(const GridC& g) { return (size_t)((g.nh - 1) / (1 << g.lb) + 1) * spec_block(g); }
 
 // A spectrum buffer with the TMA tensor maps of its y-pass and z-pass tiles.
 struct SpecBuf {
@@ -131,7 +151,7 @@ struct XVelArgs {
     const float2* G[3];       // gradient spectra (Eq. 4a, after y/z inverse)
     float* u[3];              // velocity (pitch nx)
     float2* U[3];             // XV_STEP: x-R2C of the new velocity (may alias G)
-    float* tail[3];           // XV_TAIL: u^{Nt+1/2} written as real rows of pitch 2*nhp
+    float* tail[3];           // XV_TAIL: u^{Nt+1/2} written as real rows of a spectrum buffer
     SourceC f[3];             // force sources along x, y, z (row_ptr NULL: none)
     const int64_t* step;      // device step counter (force samples)
 };
@@ -143,7 +163,7 @@ struct XDensArgs {
     float* rho[3];            // split density (pitch nx)
     float2* S;                // x-R2C of rho0 sum d  (absorbing only)
     float2* R;                // x-R2C of rho         (absorbing only)
-    float* rho_tot;           // rho as real rows of pitch 2*nhp (absorbing only)
+    float* rho_tot;           // rho as real rows of a spectrum buffer (absorbing only)
     float2* P;                // non-absorbing: x-R2C of p (EOS fused here)
     // adjoint: with keep set, the step also writes, at keep + k 7 N (k = step
     // index mod keep_period, N = nx ny nz, pitch nx): rho_xi^n as read
@@ -159,13 +179,13 @@ cudaError_t launch_x_dens(const GridC& g, const Medium& m, const SourceC& src, c
 struct XEosArgs {
     const float2* A1;         // IFT_yz{k^{y-2} ...} of S (x still spectral)
     const float2* A2;         // ... k^{y-1} of R
-    const float* rho_tot;     // pitch 2*nhp
+    const float* rho_tot;     // real rows of a spectrum buffer
     float2* P;                // x-R2C of p^{n+1}
 };
 cudaError_t launch_x_eos(const GridC& g, const Medium& m, const SourceC& dsrc, const SensorC& sens,
                          const StepC& st, const XEosArgs& a, cudaStream_t s);
 
-// plain x transforms: real rows (pitch in floats) <-> half spectra (pitch nhp)
+// plain x transforms: real rows (pitch in floats) <-> half spectra
 cudaError_t launch_x_r2c(const GridC& g, const float* in, int in_pitch, float2* out,
                          cudaStream_t s);
 cudaError_t launch_x_c2r(const GridC& g, const float2* in, float* out, int out_pitch,
@@ -175,10 +195,13 @@ cudaError_t launch_x_c2r(const GridC& g, const float2* in, float* out, int out_p
 cudaError_t launch_init_rho(const GridC& g, const Medium& m, const float* p0, int p0_pitch,
                             float* rho[3], cudaStream_t s);
 cudaError_t launch_advance_step(int64_t* step, cudaStream_t s);
+// a spectrum (16-column blocks) <-> whole rows [nz][ny][nhp], the form of a snapshot
+cudaError_t launch_spec_rows(const GridC& g, const float2* in, float2* out, bool to_rows, cudaStream_t s);
 // p_min and series sensors of one step: masked slots (p from p_sens) and u-series points
 cudaError_t launch_series(int64_t n_slots, const float* p_sens, float* p_min, const SeriesSlot* ser, float* series,
                           int64_t n_u, const int64_t* idx, const SeriesSlot* uq, float* const* u, float* useries,
                           const int64_t* step, cudaStream_t s);
+// (pitch of the u rows in floats; 0: real rows of a spectrum buffer)
 cudaError_t launch_intensity_gather(int64_t n, const int64_t* idx, const GridC& g,
                                     float* const* u, int pitch, float* ubuf, cudaStream_t s);
 cudaError_t launch_intensity_accum(int64_t n, const int64_t* idx, const GridC& g,
@@ -199,7 +222,7 @@ struct AdjX {
     // d_xi (Eq. 4c derivative), rho^{n+1}; step n's at keep + (n mod keep_period) 7 N
     const float* keep;
     int64_t keep_period;
-    float2* sp[3];            // spectra (x transformed), pitch nhp
+    float2* sp[3];            // spectra (x transformed)
     int64_t* nrev;            // reverse-step counter n, lowered by adj_x_p
 };
 // absorbing: R2C of c0^2 tau lambda_p -> sp[0] and of -c0^2 eta lambda_p -> sp[1]

@@ -162,6 +162,7 @@ extern "C" int kwgb_gradient_static(const kwgb_grid_desc* desc, int op, const fl
     g.nx = (int)n[0]; g.ny = (int)n[1]; g.nz = (int)n[2];
     g.nh = g.nx / 2 + 1;
     g.nhp = (g.nh + 15) / 16 * 16;
+    g.lb = spec_block_log2(g.nx);
     g.lognx = ilog2_static(g.nx); g.logny = ilog2_static(g.ny); g.lognz = ilog2_static(g.nz);
     g.dt = (float)desc->dt;
     g.scale = (float)(1.0 / ((double)g.nx * g.ny * g.nz));

@@ -33,6 +33,17 @@ namespace kwgb {
 
 constexpr int XTHREADS = 256;
 
+// Element k of a row's spectrum (or real row kept in a spectrum buffer); row: the
+// row's element 0 (spec_row), M: half the row length.  (The block width is a
+// constant of the row length, so that k = j + TL m costs one base and a multiple.)
+template <int M, class T>
+__device__ __forceinline__ T* spec_at(T* row, const GridC& g, int k) {
+    constexpr int LB = spec_block_log2(2 * M);
+    return row + (((size_t)g.ny * g.nz) << LB) * (k >> LB) + (k & ((1 << LB) - 1));
+}
+template <int M, class T>
+__device__ __forceinline__ T* spec_row(T* spec, int row) { return spec + ((size_t)row << spec_block_log2(2 * M)); }
+
 // Work row of a team in shared memory, and the team's barrier.
 template <int TEAM>
 struct RowSmem {
@@ -88,7 +99,7 @@ __device__ __forceinline__ float2 row_tw0(const float2* __restrict__ tw, int j) 
 // z[m] = (x[2n], x[2n+1]) with n = j + TL*m and
 // x[i] = sum_{k<nx} X[k] exp(+2 pi i k i / nx).
 template <int LOGM>
-__device__ __forceinline__ void row_c2r(const float2* __restrict__ spec, typename XShape<LOGM>::Smem& S, int j,
+__device__ __forceinline__ void row_c2r(const float2* __restrict__ spec, const GridC& g, typename XShape<LOGM>::Smem& S, int j,
                                         bool valid, const float2* __restrict__ tw,
                                         float2 (&z)[XShape<LOGM>::E]) {
     using Sh = XShape<LOGM>;
@@ -97,8 +108,8 @@ __device__ __forceinline__ void row_c2r(const float2* __restrict__ spec, typenam
     float2 t[E];
     float2 nyq = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int m = 0; m < E; ++m) t[m] = valid ? __ldcs(spec + j + TL * m) : make_float2(0.f, 0.f);
-    if (valid && j == 0) nyq = __ldcs(spec + M);
+    for (int m = 0; m < E; ++m) t[m] = valid ? __ldcs(spec_at<M>(spec, g, j + TL * m)) : make_float2(0.f, 0.f);
+    if (valid && j == 0) nyq = __ldcs(spec_at<M>(spec, g, M));
     S.sync();                                      // smem row free
 #pragma unroll
     for (int m = 0; m < E; ++m) S.at(j + TL * m) = t[m];
@@ -143,7 +154,7 @@ struct XStage {
 // stage buffer `dst` (RPT * SROW complex).  All threads of the team take part.
 template <int LOGM>
 __device__ __forceinline__ void stage_rows(float2* dst, const float2* __restrict__ spec, int first_row,
-                                           int nrows, int nhp, int lane) {
+                                           int nrows, const GridC& g, int lane) {
     using St = XStage<LOGM>;
     constexpr int CH = St::SROW / 2;                     // 16-byte chunks per row
 #pragma unroll
@@ -152,7 +163,7 @@ __device__ __forceinline__ void stage_rows(float2* dst, const float2* __restrict
         if (c < St::RPT * CH) {
             const int r = c / CH, q = c % CH;
             if (first_row + r < nrows)
-                cp_async16(dst + r * St::SROW + 2 * q, spec + (size_t)(first_row + r) * nhp + 2 * q);
+                cp_async16(dst + r * St::SROW + 2 * q, spec_at<St::M>(spec_row<St::M>(spec, first_row + r), g, 2 * q));
         }
     }
 }
@@ -182,7 +193,7 @@ __device__ __forceinline__ void row_c2r_staged(const float2* srow, typename XSha
 template <int LOGM>
 __device__ __forceinline__ void row_r2c(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
                                         bool valid, const float2* __restrict__ tw,
-                                        float2* __restrict__ spec) {
+                                        float2* __restrict__ spec, const GridC& g) {
     using Sh = XShape<LOGM>;
     constexpr int M = Sh::M, E = Sh::E, TL = Sh::TL;
     line_fft<LOGM, E, -1>(z, j, S, tw);
@@ -200,8 +211,8 @@ __device__ __forceinline__ void row_r2c(float2 (&z)[XShape<LOGM>::E], typename X
             const float2 xe = make_float2(0.5f * s.x, 0.5f * s.y);
             const float2 xo = make_float2(0.5f * d.y, -0.5f * d.x);              // d / (2i)
             const float2 x = cadd(xe, cmul(xo, row_tw<-1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
-            __stcs(spec + k, x);
-            if (k == 0) __stcs(spec + M, csub(xe, xo));
+            __stcs(spec_at<M>(spec, g, k), x);
+            if (k == 0) __stcs(spec_at<M>(spec, g, M), csub(xe, xo));
         }
     }
 }
@@ -274,7 +285,7 @@ __device__ __forceinline__ void finish_pressure(float2 (&p)[XShape<LOGM>::E], co
 
         }
     }
-    row_r2c<LOGM>(p, S, j, valid, g.t.tw, P + (size_t)row * g.nhp);
+    row_r2c<LOGM>(p, S, j, valid, g.t.tw, spec_row<Sh::M>(P, row), g);
 }
 
 // Dirichlet pressure sources of one row in step n: afterwards S.f(x) holds the

@@ -1,17 +1,21 @@
-// Instantiations of the strided-axis passes: float32 register passes.  The y
-// and z passes of 256- to 1024-point lines use the two-columns-per-thread
-// kernel (z_pair.cuh); shorter lines, and the y and absorption passes of
-// 1024-point lines, the one-column form of yz_kernel.
-#include "z_pair.cuh"
+// Instantiations of the strided-axis passes: float32 register passes.
+//
+// Lines of 64 points and more run on line_kernel (line_pass.cuh), shorter ones
+// on the one-column kernel of yz_kernel.cuh: a thread of line_kernel takes at
+// least 8 values of two columns, so a 32-point tile would be half a warp.
+// Against the kernels they replaced (8 or 16 values per thread, two exchanges
+// per transform, three for 1024 points), z_div / z_abs / y of three spectra:
+//   512^3   0.991 / 0.663 / 0.565 ms -> 0.682 / 0.439 / 0.569 ms
+//   1024^3 11.12  / 6.93  / 5.0  ms -> 6.22  / 3.76  / 4.75 ms
+//   256^3   133   / 90    / 76   us -> 91    / 59    / 78   us
+// (with the spectra in blocks of columns, kwgb_internal.h).
+#include "line_pass.cuh"
 
 namespace kwgb {
 
 template <int L, int OP>
 static cudaError_t launch_f32(const YZK& a, int items, cudaStream_t s) {
-    // (1024-point y passes and absorption pass: the one-column form measured faster;
-    // the summing divergence pass of the adjoint exists in the one-column form only)
-    if constexpr (L >= 8 && !(L == 10 && (OP == OP_Z_ABS || OP < 2)) && OP != OP_Z_DIV_SUM)
-        return launch_pair<L, OP>(a, items, s);
+    if constexpr (L >= 6) return launch_line<L, OP>(a, s);
     else return launch_t<L, OP, 0>(a, items, s);
 }
 

@@ -1,13 +1,14 @@
 #pragma once
-// Strided-axis FFT passes on the half spectra [nz][ny][nhp] (complex64).
+// Strided-axis FFT passes on the half spectra (complex64, in blocks of 16
+// columns: kwgb_internal.h).
 //
 // Work item = a tile of CX consecutive x-columns times one whole line along
 // y (y pass) or z (z pass).  The kernels are persistent: each CTA walks its
 // share of the tiles with a two-stage shared-memory ring that the TMA unit
 // fills (cp.async.bulk.tensor, box CX x 256 lines, completion on an
 // mbarrier), so the HBM reads of tile t+1 run while tile t is transformed.
-// The x extent of the tensor map is nh (not the padded pitch), so the ragged
-// last tile reads no padding: the TMA zero-fills those columns.
+// The ragged last tile reads the padding columns of the last block (zeros) and
+// stores none of them.
 //
 // Thread (c, j) takes elements j + TL*m of column c into registers; the
 // Stockham passes exchange through the stage buffer the tile arrived in, and
@@ -20,6 +21,7 @@
 // spectral multiply (Sec. 3.2): the spectrum does not return to HBM between
 // the forward and the inverse transform along z.
 #include <algorithm>
+#include <type_traits>
 
 #include "fft_core.cuh"
 #include "fft_tc.cuh"
@@ -91,6 +93,7 @@ struct alignas(64) YZK {
     int ncomp;                // y pass: components (items carry the component)
     int nloads;               // z pass: loads per item
     int load_comp[3];         // z pass: component of each load
+    int short_kappa;          // (c_ref k dt / 2)^2 <= 2 at every grid point: the short series of sinc_sq serves all
     int* flag;
 };
 
@@ -250,8 +253,9 @@ yz_kernel(const __grid_constant__ YZK a) {
         mbar_arrive_expect_tx(b, STAGE * (uint32_t)sizeof(float2) + g.wait_fault_tx);
 #pragma unroll
         for (int k = 0; k < Sh::NBOX; ++k) {
-            if (ISY) tma_load_3d(dst + k * Sh::BOX * CX, map, chunk * CX, k * Sh::BOX, line, b);
-            else tma_load_3d(dst + k * Sh::BOX * CX, map, chunk * CX, line, k * Sh::BOX, b);
+            const int x = (chunk * CX) & ((1 << g.lb) - 1), w = (chunk * CX) >> g.lb;
+            if (ISY) tma_load_4d(dst + k * Sh::BOX * CX, map, x, k * Sh::BOX, line, w, b);
+            else tma_load_4d(dst + k * Sh::BOX * CX, map, x, line, k * Sh::BOX, w, b);
         }
     };
 
@@ -294,14 +298,14 @@ yz_kernel(const __grid_constant__ YZK a) {
             const int comp = item / (nchunk * lines);
             if (!MIXED) line_fft<LOGN, E, (OP == OP_Y_FWD ? -1 : +1)>(v, j, S, g.t.tw);
             if (valid) {
-                float2* out = out_ptr(a, comp) + (size_t)line * g.ny * g.nhp + col;
+                float2* out = out_ptr(a, comp) + spec_off(g, col, 0, line);
 #pragma unroll
-                for (int m = 0; m < E; ++m) __stcs(out + (size_t)(j + TL * m) * g.nhp, v[m]);
+                for (int m = 0; m < E; ++m) __stcs(out + ((size_t)(j + TL * m) << g.lb), v[m]);
             }
         } else {
             const int y = line;
-            const size_t es = (size_t)g.ny * g.nhp;
-            const size_t off = (size_t)y * g.nhp + col;
+            const size_t es = (size_t)g.ny << g.lb;
+            const size_t off = spec_off(g, col, y, 0);
             const float kx = col < g.nh ? __ldg(g.t.kx + col) : 0.f;
             const float ky = __ldg(g.t.ky + y);
             if (l == 0) {                            // operator values of this tile, kept for its loads
