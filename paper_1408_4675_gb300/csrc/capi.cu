@@ -751,8 +751,7 @@ static void sort_by_index(std::vector<T>& v, int64_t nx, int64_t nrows) {
     v.swap(out);
 }
 
-// Row-CSR device lists of the sources of one kind (unique points per grid
-// row, each with its contributions: signal offset, length and scale sc).
+// Row-CSR device list of the sources of one kind (SourceC), scale sc.
 static int build_sources(kwgb_sim* sim, int mode, float sc, SourceC* out) {
     *out = SourceC{};
     const int64_t nx = sim->g.nx;
@@ -779,34 +778,21 @@ static int build_sources(kwgb_sim* sim, int mode, float sc, SourceC* out) {
     }
     if (!cs.empty()) {
         sort_by_index(cs, nx, nrows);
-        std::vector<int32_t> row_ptr(nrows + 1, 0), pt_x, pt_c;
-        std::vector<int64_t> c_off;
-        std::vector<int32_t> c_nt;
-        std::vector<float> c_scale;
+        std::vector<int32_t> row_ptr(nrows + 1, 0);
+        std::vector<SrcEntry> ent(cs.size());
         for (size_t i = 0; i < cs.size(); ++i) {
-            if (i == 0 || cs[i].L != cs[i - 1].L) {
-                pt_x.push_back((int32_t)(cs[i].L % nx));
-                pt_c.push_back((int32_t)c_off.size());
-                row_ptr[cs[i].L / nx + 1]++;
-            }
-            c_off.push_back(cs[i].off);
-            c_nt.push_back(cs[i].nt);
-            c_scale.push_back(sc);
+            row_ptr[cs[i].L / nx + 1]++;
+            ent[i] = SrcEntry{(int32_t)(cs[i].L % nx), cs[i].nt, cs[i].off};
         }
-        pt_c.push_back((int32_t)c_off.size());
         for (int64_t r = 0; r < nrows; ++r) row_ptr[r + 1] += row_ptr[r];
-        int32_t *d_rp, *d_px, *d_pc, *d_cnt;
-        int64_t* d_coff;
-        float *d_cs, *d_sig;
+        int32_t* d_rp;
+        SrcEntry* d_ent;
+        float* d_sig;
         if (int e = upload(sim, &d_rp, row_ptr)) return e;
-        if (int e = upload(sim, &d_px, pt_x)) return e;
-        if (int e = upload(sim, &d_pc, pt_c)) return e;
-        if (int e = upload(sim, &d_coff, c_off)) return e;
-        if (int e = upload(sim, &d_cnt, c_nt)) return e;
-        if (int e = upload(sim, &d_cs, c_scale)) return e;
+        if (int e = upload(sim, &d_ent, ent)) return e;
         if (sig.empty()) sig.push_back(0.f);
         if (int e = upload(sim, &d_sig, sig)) return e;
-        *out = SourceC{d_rp, d_px, d_pc, d_coff, d_cnt, d_cs, d_sig};
+        *out = SourceC{d_rp, d_ent, d_sig, sc};
     }
     return KWGB_OK;
 }

@@ -46,10 +46,11 @@ struct AdjXK {
 };
 
 template <int LOGM>
-__global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_absprep_kernel(const AdjXK K) {
+__global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) adj_x_absprep_kernel(const AdjXK K) {
     using Sh = XShape<LOGM>;
     constexpr int E = Sh::E, TL = Sh::TL;
     extern __shared__ float2 smem[];
+    after_previous();
     const GridC& g = K.g;
     const Medium& md = K.md;
     const int r = threadIdx.x / TL, j = threadIdx.x % TL;
@@ -77,10 +78,11 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_absprep_ke
 }
 
 template <int LOGM, bool ABS>
-__global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_dens_kernel(const AdjXK K) {
+__global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) adj_x_dens_kernel(const AdjXK K) {
     using Sh = XShape<LOGM>;
     constexpr int E = Sh::E, TL = Sh::TL;
     extern __shared__ float2 smem[];
+    after_previous();
     const GridC& g = K.g;
     const Medium& md = K.md;
     const int r = threadIdx.x / TL, j = threadIdx.x % TL;
@@ -161,10 +163,11 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_dens_kerne
 }
 
 template <int LOGM>
-__global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_vel_kernel(const AdjXK K) {
+__global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) adj_x_vel_kernel(const AdjXK K) {
     using Sh = XShape<LOGM>;
     constexpr int E = Sh::E, TL = Sh::TL;
     extern __shared__ float2 smem[];
+    after_previous();
     const GridC& g = K.g;
     const int r = threadIdx.x / TL, j = threadIdx.x % TL;
     const int nrows = g.ny * g.nz;
@@ -214,10 +217,11 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_vel_kernel
 }
 
 template <int LOGM>
-__global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) adj_x_p_kernel(const AdjXK K) {
+__global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) adj_x_p_kernel(const AdjXK K) {
     using Sh = XShape<LOGM>;
     constexpr int E = Sh::E, TL = Sh::TL;
     extern __shared__ float2 smem[];
+    after_previous();
     const GridC& g = K.g;
     const int r = threadIdx.x / TL, j = threadIdx.x % TL;
     const int row = blockIdx.x * Sh::RPB + r;
@@ -241,8 +245,9 @@ __device__ __forceinline__ float medv(const float* f, float s, int64_t i) { retu
 // The reverse step's index n is read from the device counter nrev (so that a
 // captured segment of reverse steps serves every segment), and lowered by
 // adj_x_p_kernel at the end of each reverse step.
-__global__ void adj_obj_kernel(int64_t n_obj, const int64_t* __restrict__ idx, const float* __restrict__ pobj,
-                               const int64_t* __restrict__ nrev, double weight, float* lam_p) {
+__global__ void adj_obj_kernel(int64_t n_obj, const int64_t* __restrict__ idx, const float* pobj,
+                               const int64_t* nrev, double weight, float* lam_p) {
+    after_previous();
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= n_obj) return;
     const float v = pobj[*nrev * n_obj + k];                  // p^{n+1} at objective point k
@@ -255,8 +260,9 @@ __global__ void adj_obj_kernel(int64_t n_obj, const int64_t* __restrict__ idx, c
 // scheduling (the gradient is bitwise reproducible).
 __global__ void adj_src_kernel(int rows, const int32_t* __restrict__ row_ptr, const int64_t* __restrict__ pts,
                                const float* __restrict__ scale, const int32_t* __restrict__ nt,
-                               const float* __restrict__ lam_src, Medium md, double* grad, int64_t stride,
-                               const int64_t* __restrict__ nrev) {
+                               const float* lam_src, Medium md, double* grad, int64_t stride,
+                               const int64_t* nrev) {
+    after_previous();
     const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (r >= rows) return;                                     // whole warps
     const int64_t n = *nrev;
@@ -275,7 +281,7 @@ cudaError_t launch_adj_x_absprep(const GridC& g, const Medium& m, const AdjX& a,
     AdjXK K{g, m, a};
     switch (g.lognx - 1) {
 #define CASE(L) \
-    case L: return launch_rows(adj_x_absprep_kernel<L>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s);
+    case L: return launch_rows<L>(adj_x_absprep_kernel<L>, XShape<L>::SMEM, g, K, s);
         KWGB_LOGM_CASES(CASE)
 #undef CASE
     }
@@ -287,8 +293,8 @@ cudaError_t launch_adj_x_dens(const GridC& g, const Medium& m, const AdjX& a, cu
     switch (g.lognx - 1) {
 #define CASE(L)                                                                                          \
     case L:                                                                                              \
-        if (m.absorbing) return launch_rows(adj_x_dens_kernel<L, true>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s); \
-        return launch_rows(adj_x_dens_kernel<L, false>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s);
+        if (m.absorbing) return launch_rows<L>(adj_x_dens_kernel<L, true>, XShape<L>::SMEM, g, K, s); \
+        return launch_rows<L>(adj_x_dens_kernel<L, false>, XShape<L>::SMEM, g, K, s);
         KWGB_LOGM_CASES(CASE)
 #undef CASE
     }
@@ -299,7 +305,7 @@ cudaError_t launch_adj_x_vel(const GridC& g, const Medium& m, const AdjX& a, cud
     AdjXK K{g, m, a};
     switch (g.lognx - 1) {
 #define CASE(L) \
-    case L: return launch_rows(adj_x_vel_kernel<L>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s);
+    case L: return launch_rows<L>(adj_x_vel_kernel<L>, XShape<L>::SMEM, g, K, s);
         KWGB_LOGM_CASES(CASE)
 #undef CASE
     }
@@ -310,7 +316,7 @@ cudaError_t launch_adj_x_p(const GridC& g, const Medium& m, const AdjX& a, cudaS
     AdjXK K{g, m, a};
     switch (g.lognx - 1) {
 #define CASE(L) \
-    case L: return launch_rows(adj_x_p_kernel<L>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s);
+    case L: return launch_rows<L>(adj_x_p_kernel<L>, XShape<L>::SMEM, g, K, s);
         KWGB_LOGM_CASES(CASE)
 #undef CASE
     }
@@ -320,16 +326,14 @@ cudaError_t launch_adj_x_p(const GridC& g, const Medium& m, const AdjX& a, cudaS
 cudaError_t launch_adj_obj(int64_t n_obj, const int64_t* idx, const float* pobj, const int64_t* nrev, double weight,
                            float* lam_p, cudaStream_t s) {
     if (n_obj <= 0) return cudaSuccess;
-    adj_obj_kernel<<<(unsigned)((n_obj + 255) / 256), 256, 0, s>>>(n_obj, idx, pobj, nrev, weight, lam_p);
-    return cudaGetLastError();
+    return launch_after(adj_obj_kernel, (unsigned)((n_obj + 255) / 256), 256, 0, s, n_obj, idx, pobj, nrev, weight, lam_p);
 }
 
 cudaError_t launch_adj_src(int rows, const int32_t* row_ptr, const int64_t* pts, const float* scale,
                            const int32_t* nt, const float* lam_src, const Medium& m, double* grad,
                            int64_t stride, const int64_t* nrev, cudaStream_t s) {
     if (rows <= 0) return cudaSuccess;
-    adj_src_kernel<<<(rows + 7) / 8, 256, 0, s>>>(rows, row_ptr, pts, scale, nt, lam_src, m, grad, stride, nrev);
-    return cudaGetLastError();
+    return launch_after(adj_src_kernel, (rows + 7) / 8, 256, 0, s, rows, row_ptr, pts, scale, nt, lam_src, m, grad, stride, nrev);
 }
 
 }  // namespace kwgb

@@ -4,6 +4,7 @@
 #include <cmath>
 
 #include "kwgb_internal.h"
+#include "launch.cuh"
 
 namespace kwgb {
 
@@ -62,17 +63,21 @@ cudaError_t launch_init_rho(const GridC& g, const Medium& m, const float* p0, in
     return cudaGetLastError();
 }
 
-__global__ void advance_step_kernel(int64_t* step) { *step += 1; }
+__global__ void advance_step_kernel(int64_t* step) {
+    after_previous();
+    *step += 1;
+}
 
 // Per-step work of the p_min / series sensors, after the pressure pass (which
 // leaves p^{n+1} of every masked sensor slot in p_sens): slots k < n_slots
 // update p_min and write sample n of their p series; points k < n_u write
 // u_xi^{n+1/2} into their u series.
-__global__ void series_kernel(int64_t n_slots, const float* __restrict__ p_sens, float* p_min,
+__global__ void series_kernel(int64_t n_slots, const float* p_sens, float* p_min,
                               const SeriesSlot* __restrict__ ser, float* series, int64_t n_u,
                               const int64_t* __restrict__ idx, const SeriesSlot* __restrict__ uq,
-                              const float* __restrict__ ux, const float* __restrict__ uy,
-                              const float* __restrict__ uz, float* useries, const int64_t* __restrict__ step) {
+                              const float* ux, const float* uy,
+                              const float* uz, float* useries, const int64_t* step) {
+    after_previous();
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t n = *step;
     if (k < n_slots) {
@@ -98,14 +103,12 @@ cudaError_t launch_series(int64_t n_slots, const float* p_sens, float* p_min, co
                           const int64_t* step, cudaStream_t s) {
     const int64_t n = n_slots > n_u ? n_slots : n_u;
     if (n <= 0) return cudaSuccess;
-    series_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n_slots, p_sens, p_min, ser, series, n_u, idx, uq,
+    return launch_after(series_kernel, (unsigned)((n + 255) / 256), 256, 0, s, n_slots, p_sens, p_min, ser, series, n_u, idx, uq,
                                                                u[0], u[1], u[2], useries, step);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_advance_step(int64_t* step, cudaStream_t s) {
-    advance_step_kernel<<<1, 1, 0, s>>>(step);
-    return cudaGetLastError();
+    return launch_after(advance_step_kernel, 1, 1, 0, s, step);
 }
 
 __global__ void spec_rows_kernel(GridC g, const float2* __restrict__ in, float2* __restrict__ out, bool to_rows) {
@@ -160,7 +163,8 @@ struct UPtrs {
 };
 
 __global__ void intensity_gather_kernel(int64_t n, const int64_t* __restrict__ idx, GridC g,
-                                        UPtrs u, int pitch, float* __restrict__ ubuf) {
+                                        UPtrs u, int pitch, float* ubuf) {
+    after_previous();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int64_t s = idx[i];
@@ -177,16 +181,16 @@ cudaError_t launch_intensity_gather(int64_t n, const int64_t* idx, const GridC& 
                                     float* const* u, int pitch, float* ubuf, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     UPtrs up{{u[0], u[1], u[2]}};
-    intensity_gather_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, idx, g, up, pitch, ubuf);
-    return cudaGetLastError();
+    return launch_after(intensity_gather_kernel, (unsigned)((n + 255) / 256), 256, 0, s, n, idx, g, up, pitch, ubuf);
 }
 
 // I_xi += p^n * (ubar^{n-1/2} + ubar^{n+1/2}) / 2, ubar = mean of u_xi at s - e_xi and s
 __global__ void intensity_accum_kernel(int64_t n, const int64_t* __restrict__ idx, GridC g,
-                                       UPtrs u, int pitch, const float* __restrict__ ubuf,
-                                       const float* __restrict__ p_sens,
-                                       const int32_t* __restrict__ slot, double* __restrict__ I,
-                                       const int64_t* __restrict__ step, int skip_first) {
+                                       UPtrs u, int pitch, const float* ubuf,
+                                       const float* p_sens,
+                                       const int32_t* __restrict__ slot, double* I,
+                                       const int64_t* step, int skip_first) {
+    after_previous();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (skip_first && *step == 0) return;           // p^0 is not a sample
@@ -208,9 +212,8 @@ cudaError_t launch_intensity_accum(int64_t n, const int64_t* idx, const GridC& g
                                    const int64_t* step, int skip_first, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     UPtrs up{{u[0], u[1], u[2]}};
-    intensity_accum_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, idx, g, up, pitch, ubuf,
+    return launch_after(intensity_accum_kernel, (unsigned)((n + 255) / 256), 256, 0, s, n, idx, g, up, pitch, ubuf,
                                                                        p_sens, slot, I, step, skip_first);
-    return cudaGetLastError();
 }
 
 }  // namespace kwgb

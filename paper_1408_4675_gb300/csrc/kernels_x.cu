@@ -25,7 +25,7 @@ struct XDensK {
 // density (the adjoint's recomputation).  Separate
 // instantiations, so that the common path carries no code for them.
 template <int LOGM, bool FUSED_EOS, bool DIRICHLET, bool DOUT>
-__global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_dens_kernel(const XDensK K) {
+__global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_dens_kernel(const XDensK K) {
     using Sh = XShape<LOGM>;
     using St = XStage<LOGM>;
     constexpr int E = Sh::E, TL = Sh::TL, RPW = Sh::RPT, TPB = Sh::TPB;
@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_dens_kernel(co
     const int gw = blockIdx.x * TPB + team, nw = gridDim.x * TPB;
     const int mygroups = gw < ngroups ? (ngroups - 1 - gw) / nw + 1 : 0;
 
+    after_previous();
     const size_t NN = (size_t)g.nx * g.ny * g.nz;
     float* kp = nullptr;                               // this step's kept fields
     if (DOUT) kp = K.a.keep + (size_t)(*K.st.step % K.a.keep_period) * 7 * NN;
@@ -115,17 +116,10 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_dens_kernel(co
                 for (int x = j; x < g.nx; x += TL) S.f(x) = 0.f;
             }
             S.sync();
-            for (int p = p0 + j; p < p1; p += TL) {
-                const int c0 = __ldg(K.src.pt_c + p), c1 = __ldg(K.src.pt_c + p + 1);
-                float acc = 0.f;
-                for (int c = c0; c < c1; ++c) {
-                    if (n < __ldg(K.src.c_nt + c))
-                        acc += __ldg(K.src.signal + __ldg(K.src.c_off + c) + n) * __ldg(K.src.c_scale + c);
-                }
-                const int x = __ldg(K.src.pt_x + p);
-                const float c = md.c0 ? __ldg(md.c0 + rb + x) : md.c0_s;
-                S.f(x) = __fdividef(acc, c);           // dt * 2 s / (3 c0 dx)
-            }
+            for_row_sources<TL>(K.src, p0, p1, j, n, [&](int x) { return md.c0 ? __ldg(md.c0 + rb + x) : md.c0_s; },
+                                [&](int x, float acc, bool, float c) {
+                                    S.f(x) = __fdividef(acc, c);   // dt * 2 s / (3 c0 dx)
+                                });
             S.sync();
             if (p1 > p0) {
 #pragma unroll
@@ -248,7 +242,7 @@ struct XEosStage {
 };
 
 template <int LOGM, bool DIRICHLET>
-__global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_eos_kernel(const XEosK K) {
+__global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_eos_kernel(const XEosK K) {
     using Sh = XShape<LOGM>;
     using St = XStage<LOGM>;
     using Es = XEosStage<LOGM>;
@@ -266,13 +260,9 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_eos_kernel(con
     float2* stage = smem + Sh::RPB * Sh::PITCH + team * Es::TEAM;
     const int first = blockIdx.x * Sh::RPB + team * Sh::RPT;
     const bool nl = md.nonlinear;
-    stage_rows<LOGM>(stage, K.a.A1, first, nrows, g, lane);
-    stage_rows<LOGM>(stage + Es::A, K.a.A2, first, nrows, g, lane);
-    // rho: real rows of a spectrum buffer; the medium's rows: one piece each
-    stage_real_rows<LOGM>(stage + 2 * Es::A, K.a.rho_tot, (size_t)2 << spec_block_log2(2 * M), 2 * spec_block(g), spec_block_log2(2 * M), first, nrows, lane);
+    // the medium does not depend on the kernel before: its rows are under way before the wait
     if (nl && md.rho0) stage_real_rows<LOGM>(stage + 2 * Es::A + Es::R, md.rho0, g.nx, 0, 30, first, nrows, lane);
     if (nl && md.bona) stage_real_rows<LOGM>(stage + 2 * Es::A + 2 * Es::R, md.bona, g.nx, 0, 30, first, nrows, lane);
-    cp_async_commit();
     const size_t rb = (size_t)rr * g.nx;
     const int lr = r % Sh::RPT;                          // this row within the team's stage
     // Eq. 6 with Eq. 8 and Eq. 3:
@@ -287,6 +277,13 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_eos_kernel(con
         c[m] = med2(md.c0, md.c0_s, i);
         al[m] = med2(md.alpha0, md.alpha0_s, i);
     }
+    after_previous();
+    stage_rows<LOGM>(stage, K.a.A1, first, nrows, g, lane);
+    stage_rows<LOGM>(stage + Es::A, K.a.A2, first, nrows, g, lane);
+    // rho: real rows of a spectrum buffer; the medium's rows above: one piece each
+    stage_real_rows<LOGM>(stage + 2 * Es::A, K.a.rho_tot, (size_t)2 << spec_block_log2(2 * M), 2 * spec_block(g),
+                          spec_block_log2(2 * M), first, nrows, lane);
+    cp_async_commit();
     cp_async_wait0();
     S.sync();
     const float2* cur = stage + lr * St::SROW;
@@ -346,10 +343,11 @@ struct XPlainK {
 };
 
 template <int LOGM>
-__global__ void __launch_bounds__(XTHREADS) x_r2c_kernel(const XPlainK K) {
+__global__ void __launch_bounds__(XShape<LOGM>::XT) x_r2c_kernel(const XPlainK K) {
     using Sh = XShape<LOGM>;
     constexpr int E = Sh::E, TL = Sh::TL;
     extern __shared__ float2 smem[];
+    after_previous();
     const int r = threadIdx.x / TL, j = threadIdx.x % TL;
     const int row = blockIdx.x * Sh::RPB + r;
     const bool valid = row < K.g.ny * K.g.nz;
@@ -363,10 +361,11 @@ __global__ void __launch_bounds__(XTHREADS) x_r2c_kernel(const XPlainK K) {
 }
 
 template <int LOGM>
-__global__ void __launch_bounds__(XTHREADS) x_c2r_kernel(const XPlainK K) {
+__global__ void __launch_bounds__(XShape<LOGM>::XT) x_c2r_kernel(const XPlainK K) {
     using Sh = XShape<LOGM>;
     constexpr int E = Sh::E, TL = Sh::TL;
     extern __shared__ float2 smem[];
+    after_previous();
     const int r = threadIdx.x / TL, j = threadIdx.x % TL;
     const int row = blockIdx.x * Sh::RPB + r;
     const bool valid = row < K.g.ny * K.g.nz;
@@ -412,8 +411,8 @@ cudaError_t launch_x_eos(const GridC& g, const Medium& m, const SourceC& dsrc, c
 #define CASE(L)                                                                                            \
     case L: {                                                                                              \
         const int smem = XShape<L>::SMEM + XShape<L>::TPB * XEosStage<L>::TEAM * (int)sizeof(float2);      \
-        if (dir) return launch_rows(x_eos_kernel<L, true>, XShape<L>::RPB, smem, g, K, s);                 \
-        return launch_rows(x_eos_kernel<L, false>, XShape<L>::RPB, smem, g, K, s);                         \
+        if (dir) return launch_rows<L>(x_eos_kernel<L, true>, smem, g, K, s);                 \
+        return launch_rows<L>(x_eos_kernel<L, false>, smem, g, K, s);                         \
     }
         KWGB_LOGM_CASES(CASE)
 #undef CASE
@@ -426,7 +425,7 @@ cudaError_t launch_x_r2c(const GridC& g, const float* in, int in_pitch, float2* 
     XPlainK K{g, in, in_pitch, out, nullptr, nullptr};
     switch (g.lognx - 1) {
 #define CASE(L) \
-    case L: return launch_rows(x_r2c_kernel<L>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s);
+    case L: return launch_rows<L>(x_r2c_kernel<L>, XShape<L>::SMEM, g, K, s);
         KWGB_LOGM_CASES(CASE)
 #undef CASE
     }
@@ -438,7 +437,7 @@ cudaError_t launch_x_c2r(const GridC& g, const float2* in, float* out, int out_p
     XPlainK K{g, nullptr, out_pitch, nullptr, in, out};
     switch (g.lognx - 1) {
 #define CASE(L) \
-    case L: return launch_rows(x_c2r_kernel<L>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s);
+    case L: return launch_rows<L>(x_c2r_kernel<L>, XShape<L>::SMEM, g, K, s);
         KWGB_LOGM_CASES(CASE)
 #undef CASE
     }

@@ -13,16 +13,17 @@ struct XVelK {
 };
 
 // FORCE: the launch has force sources (a separate instantiation, so that the
-// common path carries no code for them).
-template <int LOGM, int MODE, bool FORCE>
-__global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(const XVelK K) {
+// common path carries no code for them).  ONE: a CTA takes one component of its
+// rows (blockIdx mod 3) instead of all three one after another.
+template <int LOGM, int MODE, bool FORCE, bool ONE>
+__global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_vel_kernel(const XVelK K) {
     using Sh = XShape<LOGM>;
     constexpr int E = Sh::E, TL = Sh::TL;
     extern __shared__ float2 smem[];
     const GridC& g = K.g;
     const int r = threadIdx.x / TL, j = threadIdx.x % TL;
     const int nrows = g.ny * g.nz;
-    const int row = blockIdx.x * Sh::RPB + r;
+        const int row = (ONE ? blockIdx.x / 3 : blockIdx.x) * Sh::RPB + r;
     const bool valid = row < nrows;
     const int rr = valid ? row : 0;
     const int y = rr % g.ny, z = rr / g.ny;
@@ -34,31 +35,31 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(con
     float2 r0[E];                                     // rho0 of this row (x = 2n, 2n+1)
 #pragma unroll
     for (int m = 0; m < E; ++m) r0[m] = rho0 ? ldg2(rho0 + rb + 2 * (j + TL * m)) : make_float2(rho0s, rho0s);
-#pragma unroll
-    for (int xi = 0; xi < 3; ++xi) {
+    after_previous();
+    auto component = [&](int xi) {
         // issue this component's field loads before the row transform
         size_t nb;                                    // row base of the +1 neighbour along y / z
         if (xi == 1) nb = (size_t)(((y + 1) & (g.ny - 1)) + g.ny * z) * g.nx;
         else nb = (size_t)(y + g.ny * ((z + 1) & (g.nz - 1))) * g.nx;
+        float* u = pick3f(K.a.u, xi);
         float2 uo[E], r1[E];
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int x = 2 * (j + TL * m);
-            uo[m] = (MODE != XV_INIT && valid) ? ld2(K.a.u[xi] + rb + x) : make_float2(0.f, 0.f);
+            uo[m] = (MODE != XV_INIT && valid) ? ld2(u + rb + x) : make_float2(0.f, 0.f);
             if (!rho0) r1[m] = make_float2(rho0s, rho0s);
             else if (xi == 0) r1[m] = make_float2(__ldg(rho0 + rb + ((x + 2) & (g.nx - 1))), 0.f);
             else r1[m] = ldg2(rho0 + nb + x);
         }
         float2 v[E];
-        row_c2r<LOGM>(spec_row<Sh::M>(K.a.G[xi], rr), g, S, j, valid, g.t.tw, v);
+        row_c2r<LOGM>(spec_row<Sh::M>(pick3(K.a.G, xi), rr), g, S, j, valid, g.t.tw, v);
         const float fyz = xi == 1 ? __ldg(g.t.pml_sg[1] + y) : __ldg(g.t.pml_sg[2] + z);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int x = 2 * (j + TL * m);
             // staggered-grid density: mean of the two neighbours along xi
-            float2 rs;
-            if (xi == 0) rs = make_float2(0.5f * (r0[m].x + r0[m].y), 0.5f * (r0[m].y + (rho0 ? r1[m].x : rho0s)));
-            else rs = make_float2(0.5f * (r0[m].x + r1[m].x), 0.5f * (r0[m].y + r1[m].y));
+            const float2 n1 = xi == 0 ? make_float2(r0[m].y, rho0 ? r1[m].x : rho0s) : r1[m];
+            const float2 rs = make_float2(0.5f * (r0[m].x + n1.x), 0.5f * (r0[m].y + n1.y));
             const float2 f = xi == 0 ? ldg2(g.t.pml_sg[0] + x) : make_float2(fyz, fyz);
             const float2 gr = v[m];
             float2 un;
@@ -71,15 +72,15 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(con
                                  f.y * (f.y * uo[m].y - __fdividef(g.dt * gr.y, rs.y)));
             }
             if (valid) {
-                if (MODE == XV_TAIL) __stcs(spec_at<Sh::M>(spec_row<Sh::M>(reinterpret_cast<float2*>(K.a.tail[xi]), rr), g, x >> 1), un);
-                else st2(K.a.u[xi] + rb + x, un);
+                if (MODE == XV_TAIL) __stcs(spec_at<Sh::M>(spec_row<Sh::M>(reinterpret_cast<float2*>(pick3f(K.a.tail, xi)), rr), g, x >> 1), un);
+                else st2(u + rb + x, un);
             }
             v[m] = un;
         }
-        if (FORCE && MODE != XV_INIT && K.a.f[xi].row_ptr) {   // force sources along xi (uniform over the launch)
+        const SourceC& fs = xi == 0 ? K.a.f[0] : (xi == 1 ? K.a.f[1] : K.a.f[2]);
+        if (FORCE && MODE != XV_INIT && fs.row_ptr) {   // force sources along xi (uniform over the CTA)
             // u_xi += dt F / rho0_sg at the row's source points, after Eq. 4b; the
             // point's value (already stored above) is stored again by its thread
-            const SourceC& fs = K.a.f[xi];
             const int p0 = valid ? __ldg(fs.row_ptr + rr) : 0, p1 = valid ? __ldg(fs.row_ptr + rr + 1) : 0;
             S.sync();
             if (p1 > p0) {
@@ -93,24 +94,20 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(con
             S.sync();
             if (p1 > p0) {
                 const int64_t n = *K.a.step;
-                for (int p = p0 + j; p < p1; p += TL) {
-                    const int ca = __ldg(fs.pt_c + p), cb = __ldg(fs.pt_c + p + 1);
-                    float acc = 0.f;
-                    for (int c = ca; c < cb; ++c)
-                        if (n < __ldg(fs.c_nt + c)) acc += __ldg(fs.signal + __ldg(fs.c_off + c) + n) * __ldg(fs.c_scale + c);
-                    const int x = __ldg(fs.pt_x + p);
-                    float rsx = rho0s;                    // rho0 at the staggered point x + 1/2 along xi
-                    if (rho0) {
-                        const size_t other = xi == 0 ? rb + ((x + 1) & (g.nx - 1))
-                                           : xi == 1 ? (size_t)(((y + 1) & (g.ny - 1)) + g.ny * z) * g.nx + x
-                                                     : (size_t)(y + g.ny * ((z + 1) & (g.nz - 1))) * g.nx + x;
-                        rsx = 0.5f * (__ldg(rho0 + rb + x) + __ldg(rho0 + other));
-                    }
-                    const float un = S.f(x) + __fdividef(acc, rsx);
-                    S.f(x) = un;
-                    if (MODE == XV_TAIL) reinterpret_cast<float*>(spec_at<Sh::M>(spec_row<Sh::M>(reinterpret_cast<float2*>(K.a.tail[xi]), rr), g, x >> 1))[x & 1] = un;
-                    else K.a.u[xi][rb + x] = un;
-                }
+                for_row_sources<TL>(
+                    fs, p0, p1, j, n,
+                    [&](int x) {                      // rho0 at the staggered point x + 1/2 along xi
+                        if (!rho0) return rho0s;
+                        const size_t other = xi == 0 ? rb + ((x + 1) & (g.nx - 1)) : nb + x;
+                        return 0.5f * (__ldg(rho0 + rb + x) + __ldg(rho0 + other));
+                    },
+                    [&](int x, float acc, bool, float rsx) {
+                        const float un = S.f(x) + __fdividef(acc, rsx);
+                        S.f(x) = un;
+                        if (MODE == XV_TAIL)
+                            reinterpret_cast<float*>(spec_at<Sh::M>(spec_row<Sh::M>(reinterpret_cast<float2*>(pick3f(K.a.tail, xi)), rr), g, x >> 1))[x & 1] = un;
+                        else u[rb + x] = un;
+                    });
             }
             S.sync();
             if (p1 > p0) {
@@ -121,8 +118,26 @@ __global__ void __launch_bounds__(XTHREADS, XShape<LOGM>::MINB) x_vel_kernel(con
                 }
             }
         }
-        if (MODE == XV_STEP) row_r2c<LOGM>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(K.a.U[xi], rr), g);
+        if (MODE == XV_STEP) row_r2c<LOGM>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(pick3w(K.a.U, xi), rr), g);
+    };
+    if (ONE) component(blockIdx.x % 3);
+    else {
+#pragma unroll
+        for (int xi = 0; xi < 3; ++xi) component(xi);
     }
+}
+
+// All three components in one CTA read rho0 once (512^3: 1.39 ms against 1.53 ms
+// with a component per CTA).  Where those CTAs would not even fill the SMs once,
+// the components' latencies in a row are the kernel's time, and one
+// component per CTA is faster (32^3 10.2 -> 8.2 us, 32 x 256 x 128 21.4 -> 19.9 us;
+// 128^3, 1.7 times the slots: 28.9 and 27.9 us).
+template <int L, bool FORCE>
+static cudaError_t launch_step_vel(const GridC& g, const XVelK& K, cudaStream_t s) {
+    using Sh = XShape<L>;
+    const int ctas = (g.ny * g.nz + Sh::RPB - 1) / Sh::RPB;
+    if (ctas <= Sh::MINB * g.num_sms) return launch_rows<L>(x_vel_kernel<L, XV_STEP, FORCE, true>, Sh::SMEM, g, K, s, 3);
+    return launch_rows<L>(x_vel_kernel<L, XV_STEP, FORCE, false>, Sh::SMEM, g, K, s);
 }
 
 cudaError_t launch_x_vel(const GridC& g, const Medium& m, int mode, const XVelArgs& a,
@@ -132,11 +147,10 @@ cudaError_t launch_x_vel(const GridC& g, const Medium& m, int mode, const XVelAr
     switch (g.lognx - 1) {
 #define CASE(L)                                                                                   \
     case L:                                                                                       \
-        if (mode == XV_STEP && force) return launch_rows(x_vel_kernel<L, XV_STEP, true>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s); \
-        if (mode == XV_STEP) return launch_rows(x_vel_kernel<L, XV_STEP, false>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s); \
-        if (mode == XV_TAIL && force) return launch_rows(x_vel_kernel<L, XV_TAIL, true>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s); \
-        if (mode == XV_TAIL) return launch_rows(x_vel_kernel<L, XV_TAIL, false>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s); \
-        return launch_rows(x_vel_kernel<L, XV_INIT, false>, XShape<L>::RPB, XShape<L>::SMEM, g, K, s);
+        if (mode == XV_STEP) return force ? launch_step_vel<L, true>(g, K, s) : launch_step_vel<L, false>(g, K, s); \
+        if (mode == XV_TAIL && force) return launch_rows<L>(x_vel_kernel<L, XV_TAIL, true, false>, XShape<L>::SMEM, g, K, s); \
+        if (mode == XV_TAIL) return launch_rows<L>(x_vel_kernel<L, XV_TAIL, false, false>, XShape<L>::SMEM, g, K, s); \
+        return launch_rows<L>(x_vel_kernel<L, XV_INIT, false, false>, XShape<L>::SMEM, g, K, s);
         KWGB_LOGM_CASES(CASE)
 #undef CASE
     }

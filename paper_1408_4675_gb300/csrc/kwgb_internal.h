@@ -88,16 +88,19 @@ struct Medium {
     int nonlinear, absorbing;
 };
 
-// Sources: unique points per row (CSR over rows), each with a range of
-// contributions (signal row, per-point scale dt * 2 / (3 c0 dx)).
+// Sources of one kind: one entry per point and contribution, CSR over rows,
+// sorted by x within a row (entries of one point are neighbours, in the order
+// in which they were added).
+struct SrcEntry {
+    int32_t x;
+    int32_t nt;               // number of samples
+    int64_t off;              // start of the contribution's signal samples
+};
 struct SourceC {
     const int32_t* row_ptr;   // nrows + 1, NULL when there are no sources
-    const int32_t* pt_x;      // x of each unique point
-    const int32_t* pt_c;      // npts + 1 contribution ranges
-    const int64_t* c_off;     // start of the contribution's signal samples
-    const int32_t* c_nt;      // number of samples
-    const float* c_scale;     // per contribution: dt * 2 / (3 dx) (mass), dt (force), 1 (Dirichlet)
+    const SrcEntry* ent;
     const float* signal;      // all signal samples
+    float scale;              // dt * 2 / (3 dx) (mass), dt (force), 1 (Dirichlet)
 };
 
 // Masked sensor points (CSR over rows) and full-grid sensors.

@@ -456,6 +456,7 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
             else tma_load_4d(dst + k * Sh::BOX * CX, map, x, line, k * Sh::BOX, w, b);
         }
     };
+    after_previous();
     if (threadIdx.x == 0)
         for (int q = 0; q < NBUF && q < Q; ++q) issue(q);
     for (int i = grp; i < my; i += GR) {
@@ -623,8 +624,7 @@ inline cudaError_t launch_line(const YZK& a, cudaStream_t s) {
     const int units = nchunk * lines * (OP < 2 ? a.ncomp : (stash ? 1 : a.nloads));
     const int grid = std::min(a.g.num_sms, units);
     if (grid < 1) return cudaSuccess;
-    k<<<grid, 512, Ls::SMEM, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(k, grid, 512, Ls::SMEM, s, a);
 }
 
 }  // namespace kwgb

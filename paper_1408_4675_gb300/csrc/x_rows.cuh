@@ -28,10 +28,10 @@
 
 #include "fft_core.cuh"
 #include "kwgb_internal.h"
+#include "launch.cuh"
 
 namespace kwgb {
 
-constexpr int XTHREADS = 256;
 
 // Element k of a row's spectrum (or real row kept in a spectrum buffer); row: the
 // row's element 0 (spec_row), M: half the row length.  (The block width is a
@@ -64,11 +64,15 @@ struct XShape {
     static constexpr int E = M >= 8 ? 8 : M;
     static constexpr int TL = M / E;
     static constexpr int TEAM = TL > 32 ? TL : 32;   // threads of a team
+    // threads of a CTA: short rows come with small grids, where 256 threads (up to
+    // 128 rows) would leave most SMs without a CTA (32^3: 8 CTAs of 256 threads, x_vel 17.8 us and
+    // x_eos 18.4; 32 CTAs of 64: 10.2 and 14.3)
+    static constexpr int XT = LOGM <= 5 ? 64 : (LOGM <= 6 ? 128 : 256);
     static constexpr int RPT = TEAM / TL;            // rows per team
-    static constexpr int TPB = XTHREADS / TEAM;      // teams per CTA
+    static constexpr int TPB = XT / TEAM;      // teams per CTA
     static_assert(TPB >= 1 && TPB <= 15, "named barriers 1..15");
-    static constexpr int MINB = 2;                   // resident CTAs per SM the fused kernels are compiled for
-    static constexpr int RPB = XTHREADS / TL;        // rows per CTA
+    static constexpr int MINB = 512 / XT;            // resident CTAs per SM the fused kernels are compiled for
+    static constexpr int RPB = XT / TL;        // rows per CTA
     static constexpr int PITCH = M + M / 16 + 2;     // complex slots per row (padded, + Nyquist)
     static constexpr int SMEM = RPB * PITCH * (int)sizeof(float2);
     using Smem = RowSmem<TEAM>;
@@ -288,6 +292,51 @@ __device__ __forceinline__ void finish_pressure(float2 (&p)[XShape<LOGM>::E], co
     row_r2c<LOGM>(p, S, j, valid, g.t.tw, spec_row<Sh::M>(P, row), g);
 }
 
+// The source points of one row in step n, shared out over the row's TL threads:
+// f(x, sum, held, pre(x)) for each point, with the sum of its contributions
+// that still have a sample (held: there is one).  The loads of four points are
+// issued together: a row of a source plane has hundreds of them, and one after
+// another (five dependent loads each) they took longer than the row itself
+// (x_dens of a 128^3 step with a plane source 55 -> 45 us, of a 256^3 step 227 -> 185 us).
+template <int TL, class Pre, class F>
+__device__ __forceinline__ void for_row_sources(const SourceC& s, int e0, int e1, int j, int64_t n, Pre&& pre, F&& f) {
+    constexpr int U = 4;
+    for (int b = e0 + j; b < e1; b += U * TL) {
+        SrcEntry c[U];
+        int before[U], after[U];
+        float v[U], w[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int e = b + i * TL;
+            const int4 q = e < e1 ? __ldg(reinterpret_cast<const int4*>(s.ent + e)) : make_int4(-1, 0, 0, 0);
+            c[i].x = q.x;
+            c[i].nt = q.y;
+            c[i].off = (int64_t)(((uint64_t)(uint32_t)q.w << 32) | (uint32_t)q.z);
+            before[i] = e < e1 && e > e0 ? __ldg(&s.ent[e - 1].x) : -1;
+            after[i] = e + 1 < e1 ? __ldg(&s.ent[e + 1].x) : -1;
+        }
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            v[i] = n < c[i].nt ? __ldg(s.signal + c[i].off + n) * s.scale : 0.f;
+            w[i] = c[i].x >= 0 ? pre(c[i].x) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            if (c[i].x < 0 || before[i] == c[i].x) continue;        // no entry, or not the point's first
+            float acc = v[i];
+            bool held = n < c[i].nt;
+            if (after[i] == c[i].x) {
+                for (int e = b + i * TL + 1; e < e1 && __ldg(&s.ent[e].x) == c[i].x; ++e)
+                    if (n < __ldg(&s.ent[e].nt)) {
+                        acc += __ldg(s.signal + __ldg(&s.ent[e].off) + n) * s.scale;
+                        held = true;
+                    }
+            }
+            f(c[i].x, acc, held, w[i]);
+        }
+    }
+}
+
 // Dirichlet pressure sources of one row in step n: afterwards S.f(x) holds the
 // summed sample of every point x of the row that is held in this step, and
 // NaN at every other x.  All threads of the row's team call it (it contains
@@ -303,18 +352,9 @@ __device__ __forceinline__ bool dirichlet_row(const SourceC& ds, const GridC& g,
         for (int x = j; x < g.nx; x += TL) S.f(x) = __int_as_float(0x7fc00000);    // quiet NaN: not held
     }
     S.sync();
-    for (int p = p0 + j; p < p1; p += TL) {
-        const int c0 = __ldg(ds.pt_c + p), c1 = __ldg(ds.pt_c + p + 1);
-        float acc = 0.f;
-        bool held = false;
-        for (int c = c0; c < c1; ++c) {
-            if (n < __ldg(ds.c_nt + c)) {
-                acc += __ldg(ds.signal + __ldg(ds.c_off + c) + n) * __ldg(ds.c_scale + c);
-                held = true;
-            }
-        }
-        if (held) S.f(__ldg(ds.pt_x + p)) = acc;
-    }
+    for_row_sources<TL>(ds, p0, p1, j, n, [](int) { return 0.f; }, [&](int x, float acc, bool held, float) {
+        if (held) S.f(x) = acc;
+    });
     S.sync();
     return p1 > p0;
 }
@@ -334,16 +374,16 @@ __device__ __forceinline__ float2* pick3w(float2* const (&p)[3], int i) {
 }
 
 // ---------------------------------------------------------------- launchers
-template <class Kern, class Args>
-static cudaError_t launch_rows(Kern k, int rpb, int smem_bytes, const GridC& g, const Args& args,
-                               cudaStream_t s) {
+// per_row: CTAs per group of rows (x_vel: one per component)
+template <int LOGM, class Kern, class Args>
+static cudaError_t launch_rows(Kern k, int smem_bytes, const GridC& g, const Args& args, cudaStream_t s, int per_row = 1) {
+    using Sh = XShape<LOGM>;
     if (smem_bytes > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
         if (e != cudaSuccess) return e;
     }
     const int nrows = g.ny * g.nz;
-    k<<<(nrows + rpb - 1) / rpb, XTHREADS, smem_bytes, s>>>(args);
-    return cudaGetLastError();
+    return launch_after(k, (nrows + Sh::RPB - 1) / Sh::RPB * per_row, Sh::XT, smem_bytes, s, args);
 }
 
 // Persistent launch of a pipelined row kernel: one CTA per resident slot.
@@ -357,14 +397,13 @@ static cudaError_t launch_persistent(Kern k, const GridC& g, const Args& args, c
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, XTHREADS, smem_bytes);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Sh::XT, smem_bytes);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     const int ngroups = (g.ny * g.nz + Sh::RPT - 1) / Sh::RPT;
     int blocks = (ngroups + Sh::TPB - 1) / Sh::TPB;
     if (blocks > per_sm * g.num_sms) blocks = per_sm * g.num_sms;
-    k<<<blocks, XTHREADS, smem_bytes, s>>>(args);
-    return cudaGetLastError();
+    return launch_after(k, blocks, Sh::XT, smem_bytes, s, args);
 }
 
 #define KWGB_LOGM_CASES(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9)

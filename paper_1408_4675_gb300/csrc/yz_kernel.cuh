@@ -27,6 +27,7 @@
 #include "fft_tc.cuh"
 #include "fft_tc5.cuh"
 #include "kwgb_internal.h"
+#include "launch.cuh"
 #include "tma.cuh"
 
 namespace kwgb {
@@ -259,6 +260,7 @@ yz_kernel(const __grid_constant__ YZK a) {
         }
     };
 
+    after_previous();
     if (tid == 0 && Q > 0) issue(0);
     float kap[E];
     float lg[E];
@@ -466,8 +468,7 @@ inline cudaError_t launch_t(const YZK& a, int items, cudaStream_t s) {
     int grid = per_sm * a.g.num_sms;
     if (grid > items) grid = items;
     if (grid < 1) return cudaSuccess;
-    k<<<grid, Sh::THREADS, Sh::smem(MIXED), s>>>(a);
-    return cudaGetLastError();
+    return launch_after(k, grid, Sh::THREADS, Sh::smem(MIXED), s, a);
 }
 
 
