@@ -126,10 +126,11 @@ struct kwgb_sim {
         char* snap = nullptr;            // sensor accumulators after the forward run
         std::vector<std::pair<void*, size_t>> sarr;
     } adj;
-    // one captured step, replayed by kwgb_step (CUDA graph)
+    // captured steps, replayed by kwgb_step (CUDA graphs)
     cudaGraphExec_t gexec = nullptr;
+    cudaGraphExec_t gexec_n = nullptr;  // kGraphSteps steps in one graph
     cudaStream_t cap = nullptr;         // stream the step is captured on
-    int64_t glaunches = 0;              // kernels in the captured step
+    int64_t glaunches = 0;              // kernels in a captured step
     bool graph_off = false;             // capture not possible: launch directly
     bool warmed = false;                // a step has run directly (one-time set-up done)
     // per-launch event timing (kwgb_step_profiled)
@@ -569,54 +570,75 @@ static int launch_step(kwgb_sim* sim, cudaStream_t s) {
     return KWGB_OK;
 }
 
-// Capture one step into a CUDA graph (once; every launch argument of a step
-// is fixed after freeze(), and the time-dependent parts read the device step
-// counter), so that a step is one graph launch instead of 13-15 kernel
-// launches.  Called after the first step has run directly (one-time kernel
-// attribute set-up stays outside the capture).  If capture or instantiation
-// fails the simulation keeps launching kernels directly.
-static void capture_step(kwgb_sim* sim) {
-    if (sim->gexec || sim->graph_off) return;
-    sim->graph_off = true;
+// Capture `count` steps into a CUDA graph (every launch argument of a step is
+// fixed after freeze(), and the time-dependent parts read the device step
+// counter), so that a step is not 10-15 kernel launches.  Called after the first
+// step has run directly (one-time kernel attribute set-up stays outside the
+// capture).  Returns NULL if capture or instantiation fails; the simulation
+// then keeps launching kernels directly.
+static cudaGraphExec_t capture_steps(kwgb_sim* sim, int count) {
     if (!sim->cap && cudaStreamCreateWithFlags(&sim->cap, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
-        return;
+        return nullptr;
     }
     if (cudaStreamBeginCapture(sim->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
-        return;
+        return nullptr;
     }
     const int64_t l0 = sim->launches;
     const bool prof = sim->prof;
     const std::string err = sim->err;
     sim->prof = false;
-    const int e = launch_step(sim, sim->cap);
+    int e = KWGB_OK;
+    for (int i = 0; i < count && e == KWGB_OK; ++i) e = launch_step(sim, sim->cap);
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(sim->cap, &graph);
     sim->prof = prof;
-    sim->glaunches = sim->launches - l0;
+    sim->glaunches = (sim->launches - l0) / count;
     sim->launches = l0;
     sim->err = err;
-    if (e == KWGB_OK && ce == cudaSuccess && graph &&
-        cudaGraphInstantiate(&sim->gexec, graph, 0) == cudaSuccess)
-        sim->graph_off = false;
-    else
-        sim->gexec = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    if (e != KWGB_OK || ce != cudaSuccess || !graph || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) exec = nullptr;
     if (graph) cudaGraphDestroy(graph);
     cudaGetLastError();
+    return exec;
 }
 
-// One step on stream s: the captured graph when there is one, else direct launches.
-static int run_step(kwgb_sim* sim, cudaStream_t s) {
-    if (sim->warmed && !sim->prof) capture_step(sim);
-    if (sim->gexec && !sim->prof) {
-        CK(cudaGraphLaunch(sim->gexec, s));
-        sim->launches += sim->glaunches;
-        return KWGB_OK;
+// Forget the captured steps (a launch argument has changed).
+static void drop_graphs(kwgb_sim* sim) {
+    if (sim->gexec) cudaGraphExecDestroy(sim->gexec);
+    if (sim->gexec_n) cudaGraphExecDestroy(sim->gexec_n);
+    sim->gexec = sim->gexec_n = nullptr;
+}
+
+// n steps on stream s: the captured graphs when there are any, else direct launches.
+// Consecutive graph launches start on ticks of about 2 us, which is a good part of a
+// small grid's step, so runs of at least 8 kGraphSteps steps replay kGraphSteps
+// steps at a time (us per step with 1 / 4 / 8 steps a graph: 32^3 47.1 / 44.6 / 44.3, 64^3
+// 36.9 / 34.9 / 34.6); shorter runs would not pay for the second capture.
+static constexpr int kGraphSteps = 4;
+static int run_steps(kwgb_sim* sim, int64_t n, cudaStream_t s) {
+    while (n > 0) {
+        if (sim->warmed && !sim->prof && !sim->gexec && !sim->graph_off) {
+            sim->gexec = capture_steps(sim, 1);
+            sim->graph_off = sim->gexec == nullptr;
+        }
+        if (!sim->gexec || sim->prof) {
+            if (int e = launch_step(sim, s)) return e;
+            sim->warmed = true;
+            sim->steps++;
+            n--;
+            continue;
+        }
+        if (n >= 8 * kGraphSteps && !sim->gexec_n) sim->gexec_n = capture_steps(sim, kGraphSteps);
+        const bool many = n >= kGraphSteps && sim->gexec_n;
+        CK(cudaGraphLaunch(many ? sim->gexec_n : sim->gexec, s));
+        const int k = many ? kGraphSteps : 1;
+        sim->launches += k * sim->glaunches;
+        sim->steps += k;
+        n -= k;
     }
-    const int e = launch_step(sim, s);
-    if (e == KWGB_OK) sim->warmed = true;
-    return e;
+    return KWGB_OK;
 }
 
 // ------------------------------------------------------------------ initial pressure
@@ -948,11 +970,7 @@ extern "C" int kwgb_step(kwgb_sim* sim, int64_t n_steps, void* cuda_stream) {
     if (int e = freeze(sim)) return e;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     sim->last_stream = s;
-    for (int64_t i = 0; i < n_steps; ++i) {
-        if (int e = run_step(sim, s)) return e;
-        sim->steps++;
-    }
-    return KWGB_OK;
+    return run_steps(sim, n_steps, s);
 }
 
 // ------------------------------------------------------------------ checkpoint / restart
@@ -1336,10 +1354,7 @@ extern "C" int kwgb_adjoint_forward(kwgb_sim* sim, const int64_t* obj_idx, int64
     const size_t F = (size_t)sim->N * sizeof(float);
     A.keep_all = K >= n_steps;
     if (A.keep_all) {
-        if (sim->gexec) {                      // a captured step without the kept fields
-            cudaGraphExecDestroy(sim->gexec);
-            sim->gexec = nullptr;
-        }
+        drop_graphs(sim);                      // (captured without the kept fields)
         // every step's fields (7 N floats a step) instead of checkpoints: the
         // reverse pass recomputes nothing
         A.seg = static_cast<float*>(dalloc(sim, (size_t)n_steps * 7 * F));
@@ -1363,20 +1378,17 @@ extern "C" int kwgb_adjoint_forward(kwgb_sim* sim, const int64_t* obj_idx, int64
         if (!A.keep_all) return;
         sim->adj_keep = nullptr;
         sim->adj_period = 0;
-        if (sim->gexec) {
-            cudaGraphExecDestroy(sim->gexec);
-            sim->gexec = nullptr;
-        }
+        drop_graphs(sim);
     };
-    for (int64_t n = 0; n < n_steps; ++n) {
+    const int64_t run = K > 0 && !A.keep_all ? K : n_steps;
+    for (int64_t n = 0; n < n_steps; n += run) {
         int e = KWGB_OK;
-        if (K > 0 && !A.keep_all && n % K == 0) e = save_ck(sim, A.ck + (size_t)(n / K) * ck_bytes(sim), s);
-        if (!e) e = run_step(sim, s);
+        if (K > 0 && !A.keep_all) e = save_ck(sim, A.ck + (size_t)(n / K) * ck_bytes(sim), s);
+        if (!e) e = run_steps(sim, std::min(run, n_steps - n), s);
         if (e) {
             stop_keeping();
             return e;
         }
-        sim->steps++;
     }
     stop_keeping();
     if (K > 0 && !A.keep_all) {
@@ -1607,10 +1619,7 @@ extern "C" int kwgb_adjoint(kwgb_sim* sim, const int64_t* obj_idx, int64_t n_obj
 extern "C" int kwgb_debug_wait_fault(kwgb_sim* sim, int on) {
     if (!sim) return KWGB_ERR_ARG;
     sim->g.wait_fault_tx = on ? 16u : 0u;
-    if (sim->gexec) {                          // the captured step holds the old parameters
-        cudaGraphExecDestroy(sim->gexec);
-        sim->gexec = nullptr;
-    }
+    drop_graphs(sim);                          // the captured steps hold the old parameters
     sim->graph_off = false;
     return KWGB_OK;
 }
@@ -1624,7 +1633,7 @@ extern "C" const char* kwgb_last_error(const kwgb_sim* sim) {
 extern "C" void kwgb_destroy(kwgb_sim* sim) {
     if (!sim) return;
     if (sim->medium_set) cudaDeviceSynchronize();
-    if (sim->gexec) cudaGraphExecDestroy(sim->gexec);
+    drop_graphs(sim);
     if (sim->cap) cudaStreamDestroy(sim->cap);
     for (void* p : sim->allocs) {
         if (sim->freef) sim->freef(p, sim->actx);

@@ -20,6 +20,60 @@ struct XDensK {
 };
 
 
+// Additive mass source of one row (dt M_xi, identical for every xi), applied
+// after the three components: rt += 3 dt M, and rho_xi += dt M at the (few)
+// source points.  All threads of the row's team call it (it holds team barriers).
+template <int LOGM>
+__device__ __forceinline__ void mass_sources(const SourceC& src, const Medium& md, float* const (&rho)[3], const GridC& g,
+                                             const StepC& st, typename XShape<LOGM>::Smem& S, int j, bool valid, int rr,
+                                             float2 (&rt)[XShape<LOGM>::E]) {
+    constexpr int E = XShape<LOGM>::E, TL = XShape<LOGM>::TL;
+    if (!src.row_ptr) return;                          // uniform over the launch
+    const size_t rb = (size_t)rr * g.nx;
+    const int p0 = valid ? __ldg(src.row_ptr + rr) : 0;
+    const int p1 = valid ? __ldg(src.row_ptr + rr + 1) : 0;
+    const int64_t n = *st.step;
+    S.sync();
+    if (p1 > p0) {
+        for (int x = j; x < g.nx; x += TL) S.f(x) = 0.f;
+    }
+    S.sync();
+    for_row_sources<TL>(src, p0, p1, j, n, [&](int x) { return md.c0 ? __ldg(md.c0 + rb + x) : md.c0_s; },
+                        [&](int x, float acc, bool, float c) {
+                            S.f(x) = __fdividef(acc, c);   // dt * 2 s / (3 c0 dx)
+                        });
+    S.sync();
+    if (p1 > p0) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            const int x = 2 * (j + TL * m);
+            const float2 sv = make_float2(S.f(x), S.f(x + 1));
+            if (sv.x != 0.f || sv.y != 0.f) {
+#pragma unroll
+                for (int xi = 0; xi < 3; ++xi) {
+                    float* q = pick3f(rho, xi) + rb + x;
+                    float2 o = *reinterpret_cast<float2*>(q);
+                    *reinterpret_cast<float2*>(q) = make_float2(o.x + sv.x, o.y + sv.y);
+                }
+                rt[m] = make_float2(rt[m].x + 3.0f * sv.x, rt[m].y + 3.0f * sv.y);
+            }
+        }
+    }
+}
+
+// Eq. 6 without absorption at grid points i, i + 1: p = c0^2 (rho + B/2A rho^2 / rho0)
+__device__ __forceinline__ float2 eos_lossless(const Medium& md, size_t i, float2 rho) {
+    const float2 c = med2(md.c0, md.c0_s, i);
+    float2 q = rho;
+    if (md.nonlinear) {
+        const float2 ba = med2(md.bona, md.bona_s, i);
+        const float2 r0 = med2(md.rho0, md.rho0_s, i);
+        q.x += __fdividef(0.5f * ba.x * rho.x * rho.x, r0.x);
+        q.y += __fdividef(0.5f * ba.y * rho.y * rho.y, r0.y);
+    }
+    return make_float2(c.x * c.x * q.x, c.y * c.y * q.y);
+}
+
 // DIRICHLET: the launch has Dirichlet pressure sources; DOUT: it also writes
 // the Eq. 4c derivatives d_xi, the densities it read and the new total
 // density (the adjoint's recomputation).  Separate
@@ -105,39 +159,7 @@ __global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_dens_k
                 s[m] = make_float2(fmaf(r0[m].x, d[m].x, s[m].x), fmaf(r0[m].y, d[m].y, s[m].y));
             }
         }
-        // additive mass source (dt M_xi, identical for every xi), applied after the
-        // component loop: rho += 3 dt M, and rho_xi += dt M at the (few) source points
-        if (K.src.row_ptr) {                           // uniform over the launch
-            const int p0 = valid ? __ldg(K.src.row_ptr + rr) : 0;
-            const int p1 = valid ? __ldg(K.src.row_ptr + rr + 1) : 0;
-            const int64_t n = *K.st.step;
-            S.sync();
-            if (p1 > p0) {
-                for (int x = j; x < g.nx; x += TL) S.f(x) = 0.f;
-            }
-            S.sync();
-            for_row_sources<TL>(K.src, p0, p1, j, n, [&](int x) { return md.c0 ? __ldg(md.c0 + rb + x) : md.c0_s; },
-                                [&](int x, float acc, bool, float c) {
-                                    S.f(x) = __fdividef(acc, c);   // dt * 2 s / (3 c0 dx)
-                                });
-            S.sync();
-            if (p1 > p0) {
-#pragma unroll
-                for (int m = 0; m < E; ++m) {
-                    const int x = 2 * (j + TL * m);
-                    const float2 sv = make_float2(S.f(x), S.f(x + 1));
-                    if (sv.x != 0.f || sv.y != 0.f) {
-#pragma unroll
-                        for (int xi = 0; xi < 3; ++xi) {
-                            float* q = pick3f(K.a.rho, xi) + rb + x;
-                            float2 o = *reinterpret_cast<float2*>(q);
-                            *reinterpret_cast<float2*>(q) = make_float2(o.x + sv.x, o.y + sv.y);
-                        }
-                        rt[m] = make_float2(rt[m].x + 3.0f * sv.x, rt[m].y + 3.0f * sv.y);
-                    }
-                }
-            }
-        }
+        mass_sources<LOGM>(K.src, md, K.a.rho, g, K.st, S, j, valid, rr, rt);
         // Dirichlet pressure sources: rho_xi = s / (3 c0^2) at the held points
         bool drow = false;
         float2 dv[E];
@@ -169,20 +191,9 @@ __global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_dens_k
             for (int m = 0; m < E; ++m) st2(kp + 6 * NN + rb + 2 * (j + TL * m), rt[m]);
         }
         if (FUSED_EOS) {
-            // Eq. 6 without absorption: p = c0^2 (rho + B/2A rho^2 / rho0)
 #pragma unroll
             for (int m = 0; m < E; ++m) {
-                const size_t i = rb + 2 * (j + TL * m);
-                const float2 c = med2(md.c0, md.c0_s, i);
-                float2 rho = rt[m];
-                float2 q = rho;
-                if (md.nonlinear) {
-                    const float2 ba = med2(md.bona, md.bona_s, i);
-                    const float2 r0 = med2(md.rho0, md.rho0_s, i);
-                    q.x += __fdividef(0.5f * ba.x * rho.x * rho.x, r0.x);
-                    q.y += __fdividef(0.5f * ba.y * rho.y * rho.y, r0.y);
-                }
-                s[m] = make_float2(c.x * c.x * q.x, c.y * c.y * q.y);
+                s[m] = eos_lossless(md, rb + 2 * (j + TL * m), rt[m]);
                 if (DIRICHLET && drow) {                   // p = s at the held points
                     if (dv[m].x == dv[m].x) s[m].x = dv[m].x;
                     if (dv[m].y == dv[m].y) s[m].y = dv[m].y;
@@ -332,6 +343,132 @@ __global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_eos_ke
     finish_pressure<LOGM>(p, g, K.sens, K.st, S, j, valid, rr, K.a.P);
 }
 
+// ---------------------------------------------------------------- small grids
+// x_dens with the row transforms of its three spectra side by side: one warp per
+// spectrum transforms the CTA's rows (32 / TL of them) and leaves them as real rows
+// in shared memory, then the first warp, which has issued its field loads meanwhile,
+// does the pointwise work and the transform back.  For grids whose rows do not fill
+// the SMs: there the time is that of one row's chain of loads and transforms, and
+// three transforms in a row are most of it.
+template <int LOGM>
+struct XSide {
+    using Sh = XShape<LOGM>;
+    static constexpr int ROWS = 32 / Sh::TL;
+    static constexpr int smem(int spectra) { return spectra * ROWS * Sh::PITCH * (int)sizeof(float2); }
+    static_assert(Sh::TEAM == 32, "one warp holds whole rows");
+};
+
+// C2R of the warp's rows of one spectrum, left in shared memory as real rows.
+template <int LOGM>
+__device__ __forceinline__ void side_c2r(const float2* spec, const GridC& g, typename XShape<LOGM>::Smem& S, int j, bool valid, int rr) {
+    using Sh = XShape<LOGM>;
+    float2 d[Sh::E];
+    row_c2r<LOGM>(spec_row<Sh::M>(spec, rr), g, S, j, valid, g.t.tw, d);
+    S.sync();
+#pragma unroll
+    for (int m = 0; m < Sh::E; ++m) S.at(j + Sh::TL * m) = d[m];
+}
+
+template <int LOGM, bool FUSED_EOS, bool DOUT>
+__global__ void __launch_bounds__(96) x_dens_side_kernel(const XDensK K) {
+    using Sh = XShape<LOGM>;
+    constexpr int E = Sh::E, TL = Sh::TL, ROWS = XSide<LOGM>::ROWS;
+    extern __shared__ __align__(16) float2 smem[];
+    const GridC& g = K.g;
+    const Medium& md = K.md;
+    const int w = threadIdx.x / 32, r = threadIdx.x % 32 / TL, j = threadIdx.x % TL;
+    const int row = blockIdx.x * ROWS + r;
+    const bool valid = row < g.ny * g.nz;
+    const int rr = valid ? row : 0;
+    const int y = rr % g.ny, z = rr / g.ny;
+    const size_t rb = (size_t)rr * g.nx;
+    typename Sh::Smem S{smem + (w * ROWS + r) * Sh::PITCH, 0};
+    float2 r0[E];
+    if (w == 0) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) r0[m] = med2(md.rho0, md.rho0_s, rb + 2 * (j + TL * m));
+    }
+    after_previous();
+    float2 ro[3][E];
+    if (w == 0) {
+#pragma unroll
+        for (int xi = 0; xi < 3; ++xi)
+#pragma unroll
+            for (int m = 0; m < E; ++m) ro[xi][m] = valid ? ld2(K.a.rho[xi] + rb + 2 * (j + TL * m)) : make_float2(0.f, 0.f);
+    }
+    side_c2r<LOGM>(pick3(K.a.D, w), g, S, j, valid, rr);
+    __syncthreads();
+    if (w) return;
+    const size_t NN = (size_t)g.nx * g.ny * g.nz;
+    float* kp = nullptr;                               // this step's kept fields
+    if (DOUT) kp = K.a.keep + (size_t)(*K.st.step % K.a.keep_period) * 7 * NN;
+    const float fy = __ldg(g.t.pml[1] + y), fz = __ldg(g.t.pml[2] + z);
+    float2 s[E], rt[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) s[m] = rt[m] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int xi = 0; xi < 3; ++xi) {
+        typename Sh::Smem D{smem + (xi * ROWS + r) * Sh::PITCH, 0};
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            const int x = 2 * (j + TL * m);
+            const float2 d = D.at(j + TL * m);
+            const float2 f = xi == 0 ? ldg2(g.t.pml[0] + x) : (xi == 1 ? make_float2(fy, fy) : make_float2(fz, fz));
+            // Eq. 4d with the PML: rho_xi <- f (f rho_xi - dt rho0 d) / (1 + 2 dt d)
+            float2 rn = make_float2(f.x * (f.x * ro[xi][m].x - g.dt * r0[m].x * d.x), f.y * (f.y * ro[xi][m].y - g.dt * r0[m].y * d.y));
+            if (md.nonlinear) {
+                rn.x = __fdividef(rn.x, 1.0f + 2.0f * g.dt * d.x);
+                rn.y = __fdividef(rn.y, 1.0f + 2.0f * g.dt * d.y);
+            }
+            if (valid) st2(K.a.rho[xi] + rb + x, rn);
+            if (DOUT && valid) {
+                st2(kp + (3 + xi) * NN + rb + x, d);
+                st2(kp + xi * NN + rb + x, ro[xi][m]);
+            }
+            rt[m] = cadd(rt[m], rn);
+            s[m] = make_float2(fmaf(r0[m].x, d.x, s[m].x), fmaf(r0[m].y, d.y, s[m].y));
+        }
+    }
+    mass_sources<LOGM>(K.src, md, K.a.rho, g, K.st, S, j, valid, rr, rt);
+    if (DOUT && valid) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) st2(kp + 6 * NN + rb + 2 * (j + TL * m), rt[m]);
+    }
+    if (FUSED_EOS) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) s[m] = eos_lossless(md, rb + 2 * (j + TL * m), rt[m]);
+        finish_pressure<LOGM>(s, g, K.sens, K.st, S, j, valid, rr, K.a.P);
+    } else {
+        if (valid) {
+#pragma unroll
+            for (int m = 0; m < E; ++m)
+                __stcs(spec_at<Sh::M>(spec_row<Sh::M>(reinterpret_cast<float2*>(K.a.rho_tot), rr), g, j + TL * m), rt[m]);
+        }
+        row_r2c<LOGM>(s, S, j, valid, g.t.tw, spec_row<Sh::M>(K.a.S, rr), g);
+        row_r2c<LOGM>(rt, S, j, valid, g.t.tw, spec_row<Sh::M>(K.a.R, rr), g);
+    }
+}
+
+// Whether the side-by-side form serves: up to two CTAs of the plain form per SM
+// (step times: 32^3 51.0 -> 47.4 us, 64^3, 1.7 CTAs per SM, 39.1 -> 37.1; 32 x 256 x 128,
+// 3.4 CTAs per SM, 100.5 -> 102.5).  (x_eos, with two spectra, gained nothing from it.)
+template <int L>
+static bool side_by_side(const GridC& g) {
+    if constexpr (L <= 6) return (g.ny * g.nz + XShape<L>::RPB - 1) / XShape<L>::RPB <= 2 * g.num_sms;
+    else return false;
+}
+template <int L>
+static cudaError_t launch_dens_side(const GridC& g, const XDensK& K, bool fused, bool dout, cudaStream_t s) {
+    if constexpr (L <= 6) {
+        using X = XSide<L>;
+        const unsigned ctas = (g.ny * g.nz + X::ROWS - 1) / X::ROWS;
+        if (dout && fused) return launch_after(x_dens_side_kernel<L, true, true>, ctas, 96, X::smem(3), s, K);
+        if (dout) return launch_after(x_dens_side_kernel<L, false, true>, ctas, 96, X::smem(3), s, K);
+        if (fused) return launch_after(x_dens_side_kernel<L, true, false>, ctas, 96, X::smem(3), s, K);
+        return launch_after(x_dens_side_kernel<L, false, false>, ctas, 96, X::smem(3), s, K);
+    }
+    return cudaErrorInvalidValue;
+}
 // ---------------------------------------------------------------- plain x
 struct XPlainK {
     GridC g;
@@ -391,6 +528,7 @@ cudaError_t launch_x_dens(const GridC& g, const Medium& m, const SourceC& src, c
     switch (g.lognx - 1) {
 #define CASE(L)                                                                                          \
     case L:                                                                                              \
+        if (!dir && side_by_side<L>(g)) return launch_dens_side<L>(g, K, fused, dout, s);               \
         if (dout && fused) return launch_persistent<L>(x_dens_kernel<L, true, false, true>, g, K, s);   \
         if (dout) return launch_persistent<L>(x_dens_kernel<L, false, false, true>, g, K, s);           \
         if (fused && dir) return launch_persistent<L>(x_dens_kernel<L, true, true, false>, g, K, s);    \

@@ -248,23 +248,29 @@ __device__ __forceinline__ void finish_pressure(float2 (&p)[XShape<LOGM>::E], co
             float* pm = sens.full_max[k] + rbase;
             double* p2 = sens.full_p2[k] + rbase;
             float* pn = sens.full_min[k] ? sens.full_min[k] + rbase : nullptr;
+            // the row's loads before its stores: the compiler cannot tell that they do not overlap,
+            // and one after another they were eight memory latencies
+            float2 o[E];
+            double2 q[E];
+#pragma unroll
+            for (int m = 0; m < E; ++m) {
+                o[m] = *reinterpret_cast<float2*>(pm + 2 * (j + TL * m));
+                q[m] = *reinterpret_cast<double2*>(p2 + 2 * (j + TL * m));
+            }
 #pragma unroll
             for (int m = 0; m < E; ++m) {
                 const int x = 2 * (j + TL * m);
-                float2 o = *reinterpret_cast<float2*>(pm + x);
-                o.x = fmaxf(o.x, p[m].x);
-                o.y = fmaxf(o.y, p[m].y);
-                *reinterpret_cast<float2*>(pm + x) = o;
-                double2 q = *reinterpret_cast<double2*>(p2 + x);
-                q.x += (double)p[m].x * (double)p[m].x;
-                q.y += (double)p[m].y * (double)p[m].y;
-                *reinterpret_cast<double2*>(p2 + x) = q;
-                if (pn) {
-                    float2 w = *reinterpret_cast<float2*>(pn + x);
-                    w.x = fminf(w.x, p[m].x);
-                    w.y = fminf(w.y, p[m].y);
-                    *reinterpret_cast<float2*>(pn + x) = w;
-                }
+                *reinterpret_cast<float2*>(pm + x) = make_float2(fmaxf(o[m].x, p[m].x), fmaxf(o[m].y, p[m].y));
+                q[m].x += (double)p[m].x * (double)p[m].x;
+                q[m].y += (double)p[m].y * (double)p[m].y;
+                *reinterpret_cast<double2*>(p2 + x) = q[m];
+            }
+            if (pn) {
+#pragma unroll
+                for (int m = 0; m < E; ++m) o[m] = *reinterpret_cast<float2*>(pn + 2 * (j + TL * m));
+#pragma unroll
+                for (int m = 0; m < E; ++m)
+                    *reinterpret_cast<float2*>(pn + 2 * (j + TL * m)) = make_float2(fminf(o[m].x, p[m].x), fminf(o[m].y, p[m].y));
             }
         }
     }
@@ -279,14 +285,33 @@ __device__ __forceinline__ void finish_pressure(float2 (&p)[XShape<LOGM>::E], co
         S.sync();
         if (valid) {
             const int e0 = __ldg(sens.row_ptr + row), e1 = __ldg(sens.row_ptr + row + 1);
-            for (int e = e0 + j; e < e1; e += TL) {
-                const int slot = __ldg(sens.e_slot + e);
-                const float v = S.f(__ldg(sens.e_x + e));
-                sens.p_max[slot] = fmaxf(sens.p_max[slot], v);
-                sens.p2[slot] += (double)v * (double)v;
-                sens.p_sens[slot] = v;
+            // four entries at a time: a row of a sensor plane has an entry at every x (slots differ, so
+            // the order of the updates does not matter)
+            constexpr int U = 4;
+            for (int b = e0 + j; b < e1; b += U * TL) {
+                int slot[U], x[U];
+                float pm[U];
+                double p2[U];
+#pragma unroll
+                for (int i = 0; i < U; ++i) {
+                    const bool in = b + i * TL < e1;
+                    slot[i] = in ? __ldg(sens.e_slot + b + i * TL) : -1;
+                    x[i] = in ? __ldg(sens.e_x + b + i * TL) : 0;
+                }
+#pragma unroll
+                for (int i = 0; i < U; ++i) {
+                    pm[i] = slot[i] >= 0 ? sens.p_max[slot[i]] : 0.f;
+                    p2[i] = slot[i] >= 0 ? sens.p2[slot[i]] : 0.0;
+                }
+#pragma unroll
+                for (int i = 0; i < U; ++i) {
+                    if (slot[i] < 0) continue;
+                    const float v = S.f(x[i]);
+                    sens.p_max[slot[i]] = fmaxf(pm[i], v);
+                    sens.p2[slot[i]] = p2[i] + (double)v * (double)v;
+                    sens.p_sens[slot[i]] = v;
+                }
             }
-
         }
     }
     row_r2c<LOGM>(p, S, j, valid, g.t.tw, spec_row<Sh::M>(P, row), g);

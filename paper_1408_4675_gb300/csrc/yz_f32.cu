@@ -2,7 +2,9 @@
 //
 // Lines of 64 points and more run on line_kernel (line_pass.cuh), shorter ones
 // on the one-column kernel of yz_kernel.cuh: a thread of line_kernel takes at
-// least 8 values of two columns, so a 32-point tile would be half a warp.
+// least 8 values of two columns, so a 16-point tile would be half a warp, and on
+// 32-point lines its CTAs of 512 threads cost a small grid more than they save
+// (32^3 step 44.6 -> 46.1 us).
 // Against the kernels they replaced (8 or 16 values per thread, two exchanges
 // per transform, three for 1024 points), z_div / z_abs / y of three spectra:
 //   512^3   0.991 / 0.663 / 0.565 ms -> 0.682 / 0.439 / 0.569 ms
