@@ -64,14 +64,18 @@ struct XShape {
     static constexpr int E = M >= 8 ? 8 : M;
     static constexpr int TL = M / E;
     static constexpr int TEAM = TL > 32 ? TL : 32;   // threads of a team
-    // threads of a CTA: short rows come with small grids, where 256 threads (up to
-    // 128 rows) would leave most SMs without a CTA (32^3: 8 CTAs of 256 threads, x_vel 17.8 us and
-    // x_eos 18.4; 32 CTAs of 64: 10.2 and 14.3)
-    static constexpr int XT = LOGM <= 5 ? 64 : (LOGM <= 6 ? 128 : 256);
+    // threads of a CTA.  The warps of a CTA work on rows of their own, but its slot
+    // is free only when the last one has finished, and short rows come with small grids,
+    // where CTAs of 256 threads (up to 128 rows) would leave most SMs without one.  Measured:
+    // x_eos 512^3 876 -> 800 us and 1024^3 7.25 -> 6.86 ms with 128 threads instead of 256 (64: 804 us; x_vel,
+    // which reads rho0 of the rows above, 1.33 -> 1.34 ms), step 256^3 1017 -> 997 us with 64 (128: 1008),
+    // x_vel 32^3 17.8 -> 10.2 us with 64 instead of 256.
+    static constexpr int XT = LOGM <= 7 ? 64 : 128;
     static constexpr int RPT = TEAM / TL;            // rows per team
     static constexpr int TPB = XT / TEAM;      // teams per CTA
     static_assert(TPB >= 1 && TPB <= 15, "named barriers 1..15");
     static constexpr int MINB = 512 / XT;            // resident CTAs per SM the fused kernels are compiled for
+    static constexpr bool SHFL = TL <= 32;           // pairing steps by shuffles (mirrored)
     static constexpr int RPB = XT / TL;        // rows per CTA
     static constexpr int PITCH = M + M / 16 + 2;     // complex slots per row (padded, + Nyquist)
     static constexpr int SMEM = RPB * PITCH * (int)sizeof(float2);
@@ -103,7 +107,7 @@ __device__ __forceinline__ float2 row_tw0(const float2* __restrict__ tw, int j) 
 // z[m] = (x[2n], x[2n+1]) with n = j + TL*m and
 // x[i] = sum_{k<nx} X[k] exp(+2 pi i k i / nx).
 template <int LOGM>
-__device__ __forceinline__ void row_c2r(const float2* __restrict__ spec, const GridC& g, typename XShape<LOGM>::Smem& S, int j,
+__device__ __forceinline__ void row_c2r_lds(const float2* __restrict__ spec, const GridC& g, typename XShape<LOGM>::Smem& S, int j,
                                         bool valid, const float2* __restrict__ tw,
                                         float2 (&z)[XShape<LOGM>::E]) {
     using Sh = XShape<LOGM>;
@@ -129,6 +133,62 @@ __device__ __forceinline__ void row_c2r(const float2* __restrict__ spec, const G
         z[m] = make_float2(a.x - b.y, a.y + b.x);                                // a + i b
     }
     line_fft<LOGM, E, +1>(z, j, S, tw);
+}
+
+// The partner of element k in the pairing steps is element M - k: for k = j + TL m
+// that is register E - 1 - m of lane TL - j (lane 0: its own register E - m), so a
+// row within one warp gets it by a shuffle, which moves half the bytes of a round
+// trip through shared memory (x_vel is bound by that data path, 80 % busy: 512^3
+// 1.38 -> 1.33 ms, 128^3 26.4 -> 23.5 us).
+template <int TL, int E>
+__device__ __forceinline__ float2 mirrored(const float2 (&t)[E], float2 first, int j, int m) {
+    float2 o;
+    o.x = __shfl_sync(0xffffffffu, t[E - 1 - m].x, (TL - j) & (TL - 1), TL);
+    o.y = __shfl_sync(0xffffffffu, t[E - 1 - m].y, (TL - j) & (TL - 1), TL);
+    if (j == 0) o = m == 0 ? first : t[E - m > E - 1 ? 0 : E - m];
+    return o;
+}
+template <int LOGM>
+__device__ __forceinline__ void row_c2r_shfl(const float2* __restrict__ spec, const GridC& g, typename XShape<LOGM>::Smem& S, int j,
+                                             bool valid, const float2* __restrict__ tw, float2 (&z)[XShape<LOGM>::E]) {
+    using Sh = XShape<LOGM>;
+    constexpr int M = Sh::M, E = Sh::E, TL = Sh::TL;
+    float2 t[E];
+    float2 nyq = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < E; ++m) t[m] = valid ? __ldcs(spec_at<M>(spec, g, j + TL * m)) : make_float2(0.f, 0.f);
+    if (valid && j == 0) nyq = __ldcs(spec_at<M>(spec, g, M));
+    const float2 w0 = row_tw0<+1, M>(tw, j);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int k = j + TL * m;
+        const float2 xm = cconj(mirrored<TL, E>(t, nyq, j, m));
+        const float2 a = cadd(t[m], xm);
+        const float2 b = cmul(csub(t[m], xm), row_tw<+1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
+        z[m] = make_float2(a.x - b.y, a.y + b.x);                                  // a + i b
+    }
+    line_fft<LOGM, E, +1>(z, j, S, tw);
+}
+template <int LOGM>
+__device__ __forceinline__ void row_r2c_shfl(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
+                                             bool valid, const float2* __restrict__ tw, float2* __restrict__ spec, const GridC& g) {
+    using Sh = XShape<LOGM>;
+    constexpr int M = Sh::M, E = Sh::E, TL = Sh::TL;
+    line_fft<LOGM, E, -1>(z, j, S, tw);
+    const float2 w0 = row_tw0<-1, M>(tw, j);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int k = j + TL * m;
+        const float2 zm = cconj(mirrored<TL, E>(z, z[0], j, m));
+        const float2 s = cadd(z[m], zm), d = csub(z[m], zm);
+        const float2 xe = make_float2(0.5f * s.x, 0.5f * s.y);
+        const float2 xo = make_float2(0.5f * d.y, -0.5f * d.x);              // d / (2i)
+        const float2 x = cadd(xe, cmul(xo, row_tw<-1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
+        if (valid) {
+            __stcs(spec_at<M>(spec, g, k), x);
+            if (k == 0) __stcs(spec_at<M>(spec, g, M), csub(xe, xo));
+        }
+    }
 }
 
 // ---- asynchronous row staging (per-warp cp.async double buffer) ----------
@@ -193,9 +253,8 @@ __device__ __forceinline__ void row_c2r_staged(const float2* srow, typename XSha
     line_fft<LOGM, E, +1>(z, j, S, tw);
 }
 
-// Unnormalised R2C of one row: z[m] = (x[2n], x[2n+1]) -> spec[0..M].
 template <int LOGM>
-__device__ __forceinline__ void row_r2c(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
+__device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
                                         bool valid, const float2* __restrict__ tw,
                                         float2* __restrict__ spec, const GridC& g) {
     using Sh = XShape<LOGM>;
@@ -219,6 +278,22 @@ __device__ __forceinline__ void row_r2c(float2 (&z)[XShape<LOGM>::E], typename X
             if (k == 0) __stcs(spec_at<M>(spec, g, M), csub(xe, xo));
         }
     }
+}
+
+// Unnormalised R2C of one row: z[m] = (x[2n], x[2n+1]) -> spec[0..M].
+template <int LOGM>
+__device__ __forceinline__ void row_r2c(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
+                                        bool valid, const float2* __restrict__ tw,
+                                        float2* __restrict__ spec, const GridC& g) {
+    if constexpr (XShape<LOGM>::SHFL) row_r2c_shfl<LOGM>(z, S, j, valid, tw, spec, g);
+    else row_r2c_smem<LOGM>(z, S, j, valid, tw, spec, g);
+}
+
+template <int LOGM>
+__device__ __forceinline__ void row_c2r(const float2* __restrict__ spec, const GridC& g, typename XShape<LOGM>::Smem& S, int j,
+                                        bool valid, const float2* __restrict__ tw, float2 (&z)[XShape<LOGM>::E]) {
+    if constexpr (XShape<LOGM>::SHFL) row_c2r_shfl<LOGM>(spec, g, S, j, valid, tw, z);
+    else row_c2r_lds<LOGM>(spec, g, S, j, valid, tw, z);
 }
 
 __device__ __forceinline__ float2 ld2(const float* p) { return __ldcs(reinterpret_cast<const float2*>(p)); }
