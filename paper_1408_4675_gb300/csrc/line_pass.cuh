@@ -464,13 +464,30 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
         int chunk, line, l;
         place(q, chunk, line, l);
         float2* buf = smem + (q % NBUF) * Line::BUF;
+        const int ca = chunk * CX + Line::col0(c), cb = chunk * CX + Line::col1(c);
+        const bool v0 = ca < g.nh, v1 = cb < g.nh;
+        // the tile's wavenumbers and its shift operators i k e^{+-ikd/2} along x and y: under way during the wait
+        float2 kxy = dup2(0.f), xa = dup2(0.f), xb = dup2(0.f), ya = dup2(0.f);
+        if constexpr (!ISY) {
+            const float2 kx = make_float2(v0 ? __ldg(g.t.kx + ca) : 0.f, v1 ? __ldg(g.t.kx + cb) : 0.f);
+            const float ky = __ldg(g.t.ky + line);
+            if (OP != OP_Z_ABS) {
+                if (v0) xa = __ldg(g.t.dfx + ca);
+                if (v1) xb = __ldg(g.t.dfx + cb);
+                ya = __ldg(g.t.dfy + line);
+                if (BWD) {
+                    xa.x = -xa.x;
+                    xb.x = -xb.x;
+                    ya.x = -ya.x;
+                }
+            }
+            kxy = fma2(kx, kx, dup2(ky * ky));
+        }
         // A wait names a phase by its parity only, so a barrier must not be waited on before its
         // previous phase is known to be over.  Load q has barrier q mod 2 NBUF: the load before
         // on it (q - 2 NBUF) was this group's own, since GR divides 2 NBUF.
         const bool ok = mbar_wait_bounded(&bar[q % (2 * NBUF)], (q / (2 * NBUF)) & 1, a.flag);
         if (!ok) abort_flag[grp] = 1;
-        const int ca = chunk * CX + Line::col0(c), cb = chunk * CX + Line::col1(c);
-        const bool v0 = ca < g.nh, v1 = cb < g.nh;
         float2 re[H], im[H];
         // the buffer is free for its next load once every thread of the group has read it
         auto next = [&]() {
@@ -496,22 +513,7 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
             Line::template fwd_end<false>(re, im);
             const size_t es = (size_t)g.ny << g.lb;
             const size_t off = spec_off(g, ca, line, 0);
-            const float2 kx = make_float2(v0 ? __ldg(g.t.kx + ca) : 0.f, v1 ? __ldg(g.t.kx + cb) : 0.f);
-            const float ky = __ldg(g.t.ky + line);
-            const float2 kxy = fma2(kx, kx, dup2(ky * ky));
             const int comp = (OP == OP_Z_ABS && a.load_comp[0] == 1) ? 1 : l;
-            // shift operators i k e^{+-ikd/2} of the thread's columns along x, and along y
-            float2 xa = make_float2(0.f, 0.f), xb = xa, ya = xa;
-            if (OP != OP_Z_ABS) {
-                if (v0) xa = __ldg(g.t.dfx + ca);
-                if (v1) xb = __ldg(g.t.dfx + cb);
-                ya = __ldg(g.t.dfy + line);
-                if (BWD) {
-                    xa.x = -xa.x;
-                    xb.x = -xb.x;
-                    ya.x = -ya.x;
-                }
-            }
             auto dz = [&](int m, float2& zr, float2& zi) {
                 const float2 za = dfz[Line::e0(j, m)], zb = dfz[Line::e1(j, m)];
                 zr = BWD ? make_float2(-za.x, -zb.x) : make_float2(za.x, zb.x);
