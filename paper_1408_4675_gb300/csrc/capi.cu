@@ -335,8 +335,12 @@ static int build_tables(kwgb_sim* sim) {
     GridC& g = sim->g;
     const int64_t n[3] = {d.nx, d.ny, d.nz};
     const double dd[3] = {d.dx, d.dy, d.dz};
-    std::vector<float2> tw(TW_TOTAL);
-    fill_twiddle_table(tw.data());
+    // the same table for every simulation: computed once (about 11 000 sines and cosines)
+    static const std::vector<float2> tw = [] {
+        std::vector<float2> t(TW_TOTAL);
+        fill_twiddle_table(t.data());
+        return t;
+    }();
     float2* dtw;
     if (int e = upload(sim, &dtw, tw)) return e;
     g.t.tw = dtw;

@@ -162,6 +162,97 @@ __global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) adj_x_de
     }
 }
 
+// adj_x_dens with the three components side by side: warp xi of a CTA takes
+// component xi of the CTA's rows (32 / TL of them).  The plain form takes them one
+// after another, each a round of loads (the kept fields come from HBM) and a
+// transform: at 128^3 that chain is the kernel's time.
+template <int LOGM, bool ABS>
+__global__ void __launch_bounds__(96, 5) adj_x_dens_side_kernel(const AdjXK K) {
+    using Sh = XShape<LOGM>;
+    constexpr int E = Sh::E, TL = Sh::TL, ROWS = 32 / TL, M = Sh::M;
+    extern __shared__ float2 smem[];
+    after_previous();
+    const GridC& g = K.g;
+    const Medium& md = K.md;
+    const int xi = threadIdx.x / 32, r = threadIdx.x % 32 / TL, j = threadIdx.x % TL;
+    const int row = blockIdx.x * ROWS + r;
+    const bool valid = row < g.ny * g.nz;
+    const int rr = valid ? row : 0;
+    const int y = rr % g.ny, z = rr / g.ny;
+    typename Sh::Smem S{smem + (xi * ROWS + r) * Sh::PITCH, 0};
+    float2* sum = smem + 3 * ROWS * Sh::PITCH + r * M;           // component c's values at sum + c ROWS M
+    const size_t rb = (size_t)rr * g.nx;
+    const bool nl = md.nonlinear;
+    const size_t NN = (size_t)g.nx * g.ny * g.nz;
+    const float* kp = K.a.keep + (size_t)(*K.a.nrev % K.a.keep_period) * 7 * NN;   // step n's kept fields
+    float* lrho = pick3f(K.a.lam_rho, xi);
+    float2 lr[E], d[E], ro[E];                        // this component's fields: under way during the rest
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const size_t i = rb + 2 * (j + TL * m);
+        lr[m] = valid ? ld2(lrho + i) : make_float2(0.f, 0.f);
+        d[m] = valid ? ld2(kp + (3 + xi) * NN + i) : make_float2(0.f, 0.f);
+        ro[m] = valid && nl ? ld2(kp + xi * NN + i) : make_float2(0.f, 0.f);
+    }
+    if (ABS) {                                        // Eq. 8 backwards: the two C2Rs, shared through the work rows
+        if (xi < 2) {
+            float2 a[E];
+            row_c2r<LOGM>(spec_row<M>(pick3w(K.a.sp, xi), rr), g, S, j, valid, g.t.tw, a);
+            S.sync();
+#pragma unroll
+            for (int m = 0; m < E; ++m) S.at(j + TL * m) = a[m];
+        }
+        __syncthreads();
+    }
+    const float fyz = xi == 1 ? __ldg(g.t.pml[1] + y) : __ldg(g.t.pml[2] + z);
+    float2 v[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int x = 2 * (j + TL * m);
+        const size_t i = rb + x;
+        const float2 l = valid ? ld2(K.a.lam_p + i) : make_float2(0.f, 0.f);
+        const float2 c = med2(md.c0, md.c0_s, i), r0 = med2(md.rho0, md.rho0_s, i);
+        float2 w = make_float2(c.x * c.x, c.y * c.y);
+        if (nl) {                                     // dp/drho = c0^2 (1 + (B/A) rho / rho0)
+            const float2 ba = med2(md.bona, md.bona_s, i);
+            const float2 rt = valid ? ld2(kp + 6 * NN + i) : make_float2(0.f, 0.f);
+            w.x *= 1.0f + __fdividef(ba.x * rt.x, r0.x);
+            w.y *= 1.0f + __fdividef(ba.y * rt.y, r0.y);
+        }
+        float2 lrt = make_float2(w.x * l.x, w.y * l.y), labs = make_float2(0.f, 0.f);
+        if (ABS) {                                    // a1 -> lambda_d, a2 -> lambda_rho
+            const float2 a1 = smem[r * Sh::PITCH + (j + TL * m) + ((j + TL * m) >> 4)];
+            const float2 a2 = smem[(ROWS + r) * Sh::PITCH + (j + TL * m) + ((j + TL * m) >> 4)];
+            labs = make_float2(r0.x * a1.x, r0.y * a1.y);
+            lrt = cadd(lrt, a2);
+        }
+        const float2 f = xi == 0 ? ldg2(g.t.pml[0] + x) : make_float2(fyz, fyz);
+        const float2 lrp = cadd(lr[m], lrt);
+        sum[xi * ROWS * M + j + TL * m] = lrp;
+        float2 nlr;
+        if (nl) {
+            const float dx_ = __fdividef(1.0f, 1.0f + 2.0f * g.dt * d[m].x);
+            const float dy_ = __fdividef(1.0f, 1.0f + 2.0f * g.dt * d[m].y);
+            nlr = make_float2(lrp.x * f.x * f.x * dx_, lrp.y * f.y * f.y * dy_);
+            v[m] = make_float2(labs.x - lrp.x * f.x * g.dt * (r0.x + 2.0f * f.x * ro[m].x) * dx_ * dx_,
+                               labs.y - lrp.y * f.y * g.dt * (r0.y + 2.0f * f.y * ro[m].y) * dy_ * dy_);
+        } else {
+            nlr = make_float2(lrp.x * f.x * f.x, lrp.y * f.y * f.y);
+            v[m] = make_float2(labs.x - lrp.x * f.x * g.dt * r0.x, labs.y - lrp.y * f.y * g.dt * r0.y);
+        }
+        if (valid) st2(lrho + i, nlr);
+    }
+    __syncthreads();                                  // the sums' terms are written, a1 and a2 have been read
+    if (xi == 0 && valid) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            const int n = j + TL * m;
+            st2(K.a.lam_src + rb + 2 * n, cadd(cadd(sum[n], sum[ROWS * M + n]), sum[2 * ROWS * M + n]));
+        }
+    }
+    row_r2c<LOGM>(v, S, j, valid, g.t.tw, spec_row<M>(pick3w(K.a.sp, xi), rr), g);
+}
+
 template <int LOGM>
 __global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) adj_x_vel_kernel(const AdjXK K) {
     using Sh = XShape<LOGM>;
@@ -288,13 +379,27 @@ cudaError_t launch_adj_x_absprep(const GridC& g, const Medium& m, const AdjX& a,
     return cudaErrorInvalidValue;
 }
 
+// Rows within one warp (up to 512 reals): side by side (reverse pass of 128^3 x 150 steps 25.2 -> 23.6 ms,
+// 64^3 absorbing 18.3 -> 16.8, 256^3 x 16 19.2 -> 17.8, 64 x 512 x 512 x 16 20.4 -> 19.1).
+template <int L>
+static cudaError_t launch_dens(const AdjXK& K, cudaStream_t s) {
+    using Sh = XShape<L>;
+    if constexpr (Sh::TEAM == 32) {
+        constexpr int ROWS = 32 / Sh::TL, smem = 3 * ROWS * (Sh::PITCH + Sh::M) * (int)sizeof(float2);
+        const unsigned ctas = (K.g.ny * K.g.nz + ROWS - 1) / ROWS;
+        return K.md.absorbing ? launch_after(adj_x_dens_side_kernel<L, true>, ctas, 96, smem, s, K)
+                              : launch_after(adj_x_dens_side_kernel<L, false>, ctas, 96, smem, s, K);
+    } else {
+        return K.md.absorbing ? launch_rows<L>(adj_x_dens_kernel<L, true>, Sh::SMEM, K.g, K, s)
+                              : launch_rows<L>(adj_x_dens_kernel<L, false>, Sh::SMEM, K.g, K, s);
+    }
+}
+
 cudaError_t launch_adj_x_dens(const GridC& g, const Medium& m, const AdjX& a, cudaStream_t s) {
     AdjXK K{g, m, a};
     switch (g.lognx - 1) {
-#define CASE(L)                                                                                          \
-    case L:                                                                                              \
-        if (m.absorbing) return launch_rows<L>(adj_x_dens_kernel<L, true>, XShape<L>::SMEM, g, K, s); \
-        return launch_rows<L>(adj_x_dens_kernel<L, false>, XShape<L>::SMEM, g, K, s);
+#define CASE(L) \
+    case L: return launch_dens<L>(K, s);
         KWGB_LOGM_CASES(CASE)
 #undef CASE
     }
