@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_vel_ke
                 }
             }
         }
-        if (MODE == XV_STEP) row_r2c<LOGM>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(pick3w(K.a.U, xi), rr), g);
+        if (MODE == XV_STEP) row_r2c<LOGM, (LOGM >= 9)>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(pick3w(K.a.U, xi), rr), g);
     };
     if (ONE) component(blockIdx.x % 3);
     else {

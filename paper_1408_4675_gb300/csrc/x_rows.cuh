@@ -86,20 +86,19 @@ struct XShape {
     }
 };
 
-// exp(DIR 2 pi i k / (2M)) for k = j + TL*m.  Rows of 1024 reals: one table
-// load per thread (w0 = the value at k = j) times the compile-time root
-// exp(DIR i pi m / E) (TL / M = 1 / E), instead of E loads (measured faster
-// there); shorter rows: the table entry of k, loaded where it is used
-// (measured faster at 512 reals).
-template <int DIR, int M, int E>
+// exp(DIR 2 pi i k / (2M)) for k = j + TL*m.  ONE: one table load per thread (w0 =
+// the value at k = j) times the compile-time root exp(DIR i pi m / E) (TL / M = 1 / E),
+// instead of E loads.  Which is faster depends on the kernel (ms at 512^3, ONE / table: x_dens
+// 1.273 / 1.307, x_eos 0.788 / 0.806, x_vel 1.405 / 1.340; rows of 1024 reals: ONE everywhere).
+template <bool ONE, int DIR, int M, int E>
 __device__ __forceinline__ float2 row_tw(const float2* __restrict__ tw, float2 w0, int k, int m) {
     static_assert(E <= 8 && 8 % E == 0, "roots of 16");
-    if constexpr (M >= 512) return rot16<DIR>(w0, m * (8 / E));
+    if constexpr (ONE) return rot16<DIR>(w0, m * (8 / E));
     else return row_twiddle<DIR, M>(tw, k);
 }
-template <int DIR, int M>
+template <bool ONE, int DIR, int M>
 __device__ __forceinline__ float2 row_tw0(const float2* __restrict__ tw, int j) {
-    if constexpr (M >= 512) return row_twiddle<DIR, M>(tw, j);
+    if constexpr (ONE) return row_twiddle<DIR, M>(tw, j);
     else return make_float2(0.f, 0.f);
 }
 
@@ -123,13 +122,13 @@ __device__ __forceinline__ void row_c2r_lds(const float2* __restrict__ spec, con
     for (int m = 0; m < E; ++m) S.at(j + TL * m) = t[m];
     if (j == 0) S.at(M) = nyq;
     S.sync();
-    const float2 w0 = row_tw0<+1, M>(tw, j);
+    const float2 w0 = row_tw0<(M >= 512), +1, M>(tw, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int k = j + TL * m;
         const float2 xk = S.at(k), xm = cconj(S.at(M - k));
         const float2 a = cadd(xk, xm);
-        const float2 b = cmul(csub(xk, xm), row_tw<+1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
+        const float2 b = cmul(csub(xk, xm), row_tw<(M >= 512), +1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
         z[m] = make_float2(a.x - b.y, a.y + b.x);                                // a + i b
     }
     line_fft<LOGM, E, +1>(z, j, S, tw);
@@ -158,24 +157,24 @@ __device__ __forceinline__ void row_c2r_shfl(const float2* __restrict__ spec, co
 #pragma unroll
     for (int m = 0; m < E; ++m) t[m] = valid ? __ldcs(spec_at<M>(spec, g, j + TL * m)) : make_float2(0.f, 0.f);
     if (valid && j == 0) nyq = __ldcs(spec_at<M>(spec, g, M));
-    const float2 w0 = row_tw0<+1, M>(tw, j);
+    const float2 w0 = row_tw0<(M >= 512), +1, M>(tw, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int k = j + TL * m;
         const float2 xm = cconj(mirrored<TL, E>(t, nyq, j, m));
         const float2 a = cadd(t[m], xm);
-        const float2 b = cmul(csub(t[m], xm), row_tw<+1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
+        const float2 b = cmul(csub(t[m], xm), row_tw<(M >= 512), +1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
         z[m] = make_float2(a.x - b.y, a.y + b.x);                                  // a + i b
     }
     line_fft<LOGM, E, +1>(z, j, S, tw);
 }
-template <int LOGM>
+template <int LOGM, bool ONE>
 __device__ __forceinline__ void row_r2c_shfl(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
                                              bool valid, const float2* __restrict__ tw, float2* __restrict__ spec, const GridC& g) {
     using Sh = XShape<LOGM>;
     constexpr int M = Sh::M, E = Sh::E, TL = Sh::TL;
     line_fft<LOGM, E, -1>(z, j, S, tw);
-    const float2 w0 = row_tw0<-1, M>(tw, j);
+    const float2 w0 = row_tw0<ONE, -1, M>(tw, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int k = j + TL * m;
@@ -183,7 +182,7 @@ __device__ __forceinline__ void row_r2c_shfl(float2 (&z)[XShape<LOGM>::E], typen
         const float2 s = cadd(z[m], zm), d = csub(z[m], zm);
         const float2 xe = make_float2(0.5f * s.x, 0.5f * s.y);
         const float2 xo = make_float2(0.5f * d.y, -0.5f * d.x);              // d / (2i)
-        const float2 x = cadd(xe, cmul(xo, row_tw<-1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
+        const float2 x = cadd(xe, cmul(xo, row_tw<ONE, -1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
         if (valid) {
             __stcs(spec_at<M>(spec, g, k), x);
             if (k == 0) __stcs(spec_at<M>(spec, g, M), csub(xe, xo));
@@ -240,20 +239,20 @@ __device__ __forceinline__ void row_c2r_staged(const float2* srow, typename XSha
                                                float2 (&z)[XShape<LOGM>::E]) {
     using Sh = XShape<LOGM>;
     constexpr int M = Sh::M, E = Sh::E, TL = Sh::TL;
-    const float2 w0 = row_tw0<+1, M>(tw, j);
+    const float2 w0 = row_tw0<(M >= 128), +1, M>(tw, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int k = j + TL * m;
         const float2 xk = srow[k], xm = cconj(srow[M - k]);
         const float2 a = cadd(xk, xm);
-        const float2 b = cmul(csub(xk, xm), row_tw<+1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
+        const float2 b = cmul(csub(xk, xm), row_tw<(M >= 128), +1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
         z[m] = make_float2(a.x - b.y, a.y + b.x);                                // a + i b
     }
     S.sync();                                        // previous users of the work row are done
     line_fft<LOGM, E, +1>(z, j, S, tw);
 }
 
-template <int LOGM>
+template <int LOGM, bool ONE>
 __device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
                                         bool valid, const float2* __restrict__ tw,
                                         float2* __restrict__ spec, const GridC& g) {
@@ -265,7 +264,7 @@ __device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typen
     for (int m = 0; m < E; ++m) S.at(j + TL * m) = z[m];
     S.sync();
     if (valid) {
-        const float2 w0 = row_tw0<-1, M>(tw, j);
+        const float2 w0 = row_tw0<ONE, -1, M>(tw, j);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int k = j + TL * m;
@@ -273,7 +272,7 @@ __device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typen
             const float2 s = cadd(zk, zm), d = csub(zk, zm);
             const float2 xe = make_float2(0.5f * s.x, 0.5f * s.y);
             const float2 xo = make_float2(0.5f * d.y, -0.5f * d.x);              // d / (2i)
-            const float2 x = cadd(xe, cmul(xo, row_tw<-1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
+            const float2 x = cadd(xe, cmul(xo, row_tw<ONE, -1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
             __stcs(spec_at<M>(spec, g, k), x);
             if (k == 0) __stcs(spec_at<M>(spec, g, M), csub(xe, xo));
         }
@@ -281,12 +280,12 @@ __device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typen
 }
 
 // Unnormalised R2C of one row: z[m] = (x[2n], x[2n+1]) -> spec[0..M].
-template <int LOGM>
+template <int LOGM, bool ONE = (LOGM >= 7)>
 __device__ __forceinline__ void row_r2c(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
                                         bool valid, const float2* __restrict__ tw,
                                         float2* __restrict__ spec, const GridC& g) {
-    if constexpr (XShape<LOGM>::SHFL) row_r2c_shfl<LOGM>(z, S, j, valid, tw, spec, g);
-    else row_r2c_smem<LOGM>(z, S, j, valid, tw, spec, g);
+    if constexpr (XShape<LOGM>::SHFL) row_r2c_shfl<LOGM, ONE>(z, S, j, valid, tw, spec, g);
+    else row_r2c_smem<LOGM, ONE>(z, S, j, valid, tw, spec, g);
 }
 
 template <int LOGM>
