@@ -449,12 +449,14 @@ __global__ void __launch_bounds__(96) x_dens_side_kernel(const XDensK K) {
     }
 }
 
-// Whether the side-by-side form serves: up to two CTAs of the plain form per SM
-// (step times: 32^3 51.0 -> 47.4 us, 64^3, 1.7 CTAs per SM, 39.1 -> 37.1; 32 x 256 x 128,
-// 3.4 CTAs per SM, 100.5 -> 102.5).  (x_eos, with two spectra, gained nothing from it.)
+// Whether the side-by-side form serves, by the plain form's CTAs per SM: up to two in an
+// absorbing medium (step times: 32^3 51.0 -> 47.4 us; 32 x 256 x 128, 6.7 CTAs, 100.5 -> 102.5),
+// up to 16 in a lossless one, whose first warp has one transform back instead of two
+// (64^3 39.1 -> 37.1 us, 128^3, 13.5 CTAs, 108.3 -> 106.6).  (x_eos, with two spectra, gained
+// nothing from it.)
 template <int L>
-static bool side_by_side(const GridC& g) {
-    if constexpr (L <= 6) return (g.ny * g.nz + XShape<L>::RPB - 1) / XShape<L>::RPB <= 2 * g.num_sms;
+static bool side_by_side(const GridC& g, bool absorbing) {
+    if constexpr (L <= 6) return (g.ny * g.nz + XShape<L>::RPB - 1) / XShape<L>::RPB <= (absorbing ? 2 : 16) * g.num_sms;
     else return false;
 }
 template <int L>
@@ -528,7 +530,7 @@ cudaError_t launch_x_dens(const GridC& g, const Medium& m, const SourceC& src, c
     switch (g.lognx - 1) {
 #define CASE(L)                                                                                          \
     case L:                                                                                              \
-        if (!dir && side_by_side<L>(g)) return launch_dens_side<L>(g, K, fused, dout, s);               \
+        if (!dir && side_by_side<L>(g, !fused)) return launch_dens_side<L>(g, K, fused, dout, s);               \
         if (dout && fused) return launch_persistent<L>(x_dens_kernel<L, true, false, true>, g, K, s);   \
         if (dout) return launch_persistent<L>(x_dens_kernel<L, false, false, true>, g, K, s);           \
         if (fused && dir) return launch_persistent<L>(x_dens_kernel<L, true, true, false>, g, K, s);    \

@@ -359,9 +359,9 @@ __device__ __forceinline__ void finish_pressure(float2 (&p)[XShape<LOGM>::E], co
         S.sync();
         if (valid) {
             const int e0 = __ldg(sens.row_ptr + row), e1 = __ldg(sens.row_ptr + row + 1);
-            // four entries at a time: a row of a sensor plane has an entry at every x (slots differ, so
+            // U entries at a time: a row of a sensor plane has an entry at every x (slots differ, so
             // the order of the updates does not matter)
-            constexpr int U = 4;
+            constexpr int U = TL <= 8 ? 8 : 4;
             for (int b = e0 + j; b < e1; b += U * TL) {
                 int slot[U], x[U];
                 float pm[U];
@@ -393,13 +393,13 @@ __device__ __forceinline__ void finish_pressure(float2 (&p)[XShape<LOGM>::E], co
 
 // The source points of one row in step n, shared out over the row's TL threads:
 // f(x, sum, held, pre(x)) for each point, with the sum of its contributions
-// that still have a sample (held: there is one).  The loads of four points are
+// that still have a sample (held: there is one).  The loads of U points are
 // issued together: a row of a source plane has hundreds of them, and one after
 // another (five dependent loads each) they took longer than the row itself
 // (x_dens of a 128^3 step with a plane source 55 -> 45 us, of a 256^3 step 227 -> 185 us).
 template <int TL, class Pre, class F>
 __device__ __forceinline__ void for_row_sources(const SourceC& s, int e0, int e1, int j, int64_t n, Pre&& pre, F&& f) {
-    constexpr int U = 4;
+    constexpr int U = TL <= 8 ? 8 : 4;
     for (int b = e0 + j; b < e1; b += U * TL) {
         SrcEntry c[U];
         int before[U], after[U];
