@@ -168,6 +168,9 @@ extern "C" int kwgb_gradient_static(const kwgb_grid_desc* desc, int op, const fl
     g.scale = (float)(1.0 / ((double)g.nx * g.ny * g.nz));
     g.hk = (float)(desc->c_ref * desc->dt / 2.0);
     g.hk2 = (float)((desc->c_ref * desc->dt / 2.0) * (desc->c_ref * desc->dt / 2.0));
+    double kmax2 = 0;
+    for (int a = 0; a < 3; ++a) kmax2 += (kPi / dd[a]) * (kPi / dd[a]);
+    g.inv_kmax2 = (float)(1.0 / kmax2);   // (whether the short kappa series serves every point)
     g.num_sms = sms;
 
     {
