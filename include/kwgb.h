@@ -197,9 +197,10 @@ int kwgb_set_series_capacity(kwgb_sim* sim, int32_t sensor_id, int64_t n_t);
  * indices grouped by grid row on the host, uploaded, one device
  * synchronisation); from then on sources and sensors are fixed.
  * The first step of a simulation launches its kernels directly and the
- * library then captures one step into a CUDA graph (on a stream of its own)
- * that later steps replay on cuda_stream; if capture is not possible the
- * kernels keep being launched directly.  Either way the results are the
+ * library then captures the step into CUDA graphs (one step, and four steps
+ * once a call has 32 or more left; on a stream of its own) that later steps
+ * replay on cuda_stream; if capture is not possible the kernels keep being
+ * launched directly.  Either way the results are the
  * same.  Errors: ARG (n_steps < 0), STATE (no medium), CUDA. */
 int kwgb_step(kwgb_sim* sim, int64_t n_steps, void* cuda_stream);
 
@@ -247,7 +248,7 @@ int kwgb_apply_operator(kwgb_sim* sim, int op, const float* in, float* out0,
  *   err       optional buffer (errlen bytes) that receives a message on failure
  * Asynchronous on cuda_stream.  It allocates nothing and calls no cudaMalloc
  * or cudaFree: its scratch (three spectra and small tables) is one file-scope
- * device array of about 4.7 MB that every GPU loading the library's device
+ * device array of about 4.8 MB that every GPU loading the library's device
  * code holds until the process exits.  Larger grids are rejected with
  * KWGB_ERR_UNSUPPORTED.
  * The first call on a device does the set-up: under CUDA's lazy module

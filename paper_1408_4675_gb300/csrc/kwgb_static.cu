@@ -6,7 +6,7 @@
 // code paths that must not allocate after initialisation, because cudaMalloc
 // can synchronise the device and can fail once memory has been committed
 // elsewhere.  This entry point therefore takes its scratch space from one
-// file-scope __device__ array instead of allocating: about 4.7 MB, enough for
+// file-scope __device__ array instead of allocating: about 4.8 MB, enough for
 // grids up to 64 x 64 x 64, which every GPU that loads the library's device
 // code holds until the process exits.  With CUDA's lazy module loading that
 // code (and the array) is loaded on the first call on each device, so that
