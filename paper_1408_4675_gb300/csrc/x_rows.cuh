@@ -44,17 +44,23 @@ __device__ __forceinline__ T* spec_at(T* row, const GridC& g, int k) {
 template <int M, class T>
 __device__ __forceinline__ T* spec_row(T* spec, int row) { return spec + ((size_t)row << spec_block_log2(2 * M)); }
 
-// Work row of a team in shared memory, and the team's barrier.
-template <int TEAM>
+// Work row of a team in shared memory, and the team's barrier.  TEAMS: teams per CTA.
+// The barrier ids are literals: with an id in a register the compiler reserves all 16 barriers
+// for a CTA, and the SM's barriers then limit how many of the small CTAs of the plain
+// x transforms it holds (gradient of 256 x 512 x 1024, three literal barriers instead of 16:
+// 2.22 -> 1.95 ms, eta of 64 x 512 x 1024 258 -> 226 us, step of 1024^3 65.3 -> 64.8 ms).
+template <int TEAM, int TEAMS>
 struct RowSmem {
     float2* base;
-    int bar;                                         // named barrier id (TEAM > 32)
+    int team;                                        // this team (TEAM > 32)
     static constexpr bool PINGPONG = false;
     __device__ __forceinline__ float2& at(int e) { return base[e + (e >> 4)]; }
     __device__ __forceinline__ float& f(int x) { return reinterpret_cast<float*>(base)[x]; }
     __device__ __forceinline__ void sync() {
+        static_assert(TEAM <= 32 || TEAMS == 2, "one barrier per team");
         if constexpr (TEAM <= 32) __syncwarp();
-        else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(TEAM) : "memory");
+        else if (team == 0) asm volatile("bar.sync 1, %0;" ::"n"(TEAM) : "memory");
+        else asm volatile("bar.sync 2, %0;" ::"n"(TEAM) : "memory");
     }
 };
 
@@ -73,16 +79,16 @@ struct XShape {
     static constexpr int XT = LOGM <= 7 ? 64 : 128;
     static constexpr int RPT = TEAM / TL;            // rows per team
     static constexpr int TPB = XT / TEAM;      // teams per CTA
-    static_assert(TPB >= 1 && TPB <= 15, "named barriers 1..15");
+    static_assert(TPB >= 1, "a CTA holds whole teams");
     static constexpr int MINB = 512 / XT;            // resident CTAs per SM the fused kernels are compiled for
     static constexpr bool SHFL = TL <= 32;           // pairing steps by shuffles (mirrored)
     static constexpr int RPB = XT / TL;        // rows per CTA
     static constexpr int PITCH = M + M / 16 + 2;     // complex slots per row (padded, + Nyquist)
     static constexpr int SMEM = RPB * PITCH * (int)sizeof(float2);
-    using Smem = RowSmem<TEAM>;
+    using Smem = RowSmem<TEAM, TPB>;
     // the work row of row slot r (threads r*TL .. r*TL + TL - 1) of a CTA
     __device__ __forceinline__ static Smem row_smem(float2* smem, int r) {
-        return Smem{smem + r * PITCH, 1 + (r * TL) / TEAM};
+        return Smem{smem + r * PITCH, (r * TL) / TEAM};
     }
 };
 
