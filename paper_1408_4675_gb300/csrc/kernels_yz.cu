@@ -24,22 +24,36 @@ static EncodeTiledFn encode_fn() {
     return fn;
 }
 
+// The last block of a spectrum is never full (nx/2 + 1 columns).  In a spectrum of 64 MB and
+// more its tiles come through a tensor map of their own, which ends with the last column and
+// promotes no fetch, so that the padding beside it stays in HBM: at 512 x 512 x 128 the forward
+// y pass of one spectrum reads 206 MB with the 256-byte pieces, 172 without (136 are needed: the Nyquist column's
+// sectors bring their 128-byte lines), at 1024 x 1024 x 128 896 and 730.  Steps: 1024 x 1024 x 128
+// 9.06 -> 8.62 ms, 512^3 7.54 -> 7.45, 512 x 1024 x 8 0.81 -> 0.72.  Smaller spectra stay in L2, where the
+// padding costs nothing and the clipped map does (512 x 512 x 16, 34 MB, 455 -> 469 us).
+static bool clips_last_block(const GridC& g) { return spec_elems(g) * sizeof(float2) >= (size_t)64 << 20; }
+
+// map[0]: every block at its full width; map[1]: the last one up to the last column
 template <int LOGN, bool ISY, int MIXED>
-static int encode_box(const GridC& g, float2* ptr, CUtensorMap* map) {
+static int encode_box(const GridC& g, float2* ptr, CUtensorMap (&map)[2]) {
     using Sh = TShape<LOGN, ISY, MIXED>;
     EncodeTiledFn fn = encode_fn();
     if (!fn) return -1;
-    // 16-column blocks: a tile's CX columns lie in one block (CX divides 16)
+    // a tile's CX columns lie in one block (CX divides the block width, 16 or 32)
     static_assert(16 % Sh::CX == 0, "tile width");
-    const cuuint64_t w = (cuuint64_t)1 << g.lb, row = w * 8;
-    const cuuint64_t dims[4] = {w, (cuuint64_t)g.ny, (cuuint64_t)g.nz, (g.nh + w - 1) / w};
+    const cuuint64_t w = (cuuint64_t)1 << g.lb, row = w * 8, full = (g.nh - 1) / w;
     const cuuint64_t strides[3] = {row, g.ny * row, (cuuint64_t)g.ny * g.nz * row};
     const cuuint32_t box[4] = {(cuuint32_t)Sh::CX, ISY ? (cuuint32_t)Sh::BOX : 1u, ISY ? 1u : (cuuint32_t)Sh::BOX, 1u};
     const cuuint32_t es[4] = {1, 1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 4, ptr, dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? 0 : -2;
+    for (int last = 0; last < 2; ++last) {
+        const cuuint64_t dims[4] = {last ? g.nh - full * w : w, (cuuint64_t)g.ny, (cuuint64_t)g.nz, last ? 1 : full + 1};
+        const CUresult r = fn(&map[last], CU_TENSOR_MAP_DATA_TYPE_INT64, 4, ptr + (last ? full * spec_block(g) : 0), dims,
+                              strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                              last ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return -2;
+    }
+    return 0;
 }
 
 
@@ -47,13 +61,13 @@ int make_spec_maps(const GridC& g, float2* ptr, SpecBuf* out) {
     out->p = ptr;
     int e = -3;
     switch (g.logny) {
-#define CASE(L) case L: e = g.mixed ? encode_box<L, true, 1>(g, ptr, &out->ymap) : encode_box<L, true, 0>(g, ptr, &out->ymap); break;
+#define CASE(L) case L: e = g.mixed ? encode_box<L, true, 1>(g, ptr, out->ymap) : encode_box<L, true, 0>(g, ptr, out->ymap); break;
         KWGB_LOG_CASES(CASE)
 #undef CASE
     }
     if (e) return e;
     switch (g.lognz) {
-#define CASE(L) case L: e = g.mixed ? encode_box<L, false, 1>(g, ptr, &out->zmap) : encode_box<L, false, 0>(g, ptr, &out->zmap); break;
+#define CASE(L) case L: e = g.mixed ? encode_box<L, false, 1>(g, ptr, out->zmap) : encode_box<L, false, 0>(g, ptr, out->zmap); break;
         KWGB_LOG_CASES(CASE)
 #undef CASE
     }
@@ -64,6 +78,11 @@ static cudaError_t launch_op(int op, const YZK& a, int logn, int items, cudaStre
     if (a.g.mixed == 2) return yz_dispatch_f16(a, op, logn, items, s);
     if (a.g.mixed == 1) return yz_dispatch_bf16(a, op, logn, items, s);
     return yz_dispatch_f32(a, op, logn, items, s);
+}
+
+static void set_maps(YZK& a, int i, const CUtensorMap (&m)[2]) {
+    a.map[i] = m[0];
+    a.map[3 + i] = m[1];
 }
 
 static int chunk_count(int nh, int cx) { return (nh + cx - 1) / cx; }
@@ -85,12 +104,13 @@ cudaError_t launch_y_pass(const GridC& g, int dir, const SpecBuf* const* in, flo
     memset(&a, 0, sizeof(a));
     a.g = g;
     for (int i = 0; i < ncomp; ++i) {
-        a.map[i] = in[i]->ymap;
+        set_maps(a, i, in[i]->ymap);
         a.out[i] = out[i];
     }
     a.ncomp = ncomp;
     a.nloads = 1;
     a.flag = flag;
+    a.clip = clips_last_block(g) ? (g.nh - 1) >> g.lb : -1;
     const int items = chunk_count(g.nh, cx_of<true>(g.logny, g.mixed)) * g.nz * ncomp;
     return launch_op(dir < 0 ? OP_Y_FWD : OP_Y_INV, a, g.logny, items, s);
 }
@@ -101,15 +121,16 @@ cudaError_t launch_z_op(const GridC& g, int kind, const SpecBuf* const* in, floa
     memset(&a, 0, sizeof(a));
     a.g = g;
     a.flag = flag;
+    a.clip = clips_last_block(g) ? (g.nh - 1) >> g.lb : -1;
     for (int i = 0; i < 3; ++i) a.out[i] = out[i];
     a.short_kappa = g.hk2 <= 1.9999f * g.inv_kmax2;   // with room for the rounding of k^2
     if (kind == Z_GRAD_FWD || kind == Z_GRAD_BWD) {
-        a.map[0] = in[0]->zmap;
+        set_maps(a, 0, in[0]->zmap);
         a.nloads = 1;
         a.load_comp[0] = 0;
     } else if (kind == Z_DIV || kind == Z_DIV_FWD || kind == Z_DIV_SUM) {
         for (int i = 0; i < 3; ++i) {
-            a.map[i] = in[i]->zmap;
+            set_maps(a, i, in[i]->zmap);
             a.load_comp[i] = i;
         }
         a.nloads = 3;
@@ -117,7 +138,7 @@ cudaError_t launch_z_op(const GridC& g, int kind, const SpecBuf* const* in, floa
         int n = 0;
         for (int t = 0; t < 2; ++t)
             if (in[t]) {
-                a.map[t] = in[t]->zmap;
+                set_maps(a, t, in[t]->zmap);
                 a.load_comp[n++] = t;
             }
         a.nloads = n;

@@ -68,13 +68,14 @@ __host__ __device__ inline size_t spec_off(const GridC& g, int col, int y, int z
 }
 inline size_t spec_elems(const GridC& g) { return (size_t)((g.nh - 1) / (1 << g.lb) + 1) * spec_block(g); }
 
-// A spectrum buffer with the TMA tensor maps of its y-pass and z-pass tiles.
+// A spectrum buffer with the TMA tensor maps of its y-pass and z-pass tiles: [0]
+// every block of columns, [1] the last block up to the last column.
 struct SpecBuf {
     float2* p;
-    CUtensorMap ymap;
-    CUtensorMap zmap;
+    CUtensorMap ymap[2];
+    CUtensorMap zmap[2];
 };
-// Encode the two tensor maps of a spectrum buffer (0 on success).
+// Encode the tensor maps of a spectrum buffer (0 on success).
 int make_spec_maps(const GridC& g, float2* ptr, SpecBuf* out);
 
 struct Medium {
@@ -198,7 +199,7 @@ cudaError_t launch_x_c2r(const GridC& g, const float2* in, float* out, int out_p
 cudaError_t launch_init_rho(const GridC& g, const Medium& m, const float* p0, int p0_pitch,
                             float* rho[3], cudaStream_t s);
 cudaError_t launch_advance_step(int64_t* step, cudaStream_t s);
-// a spectrum (16-column blocks) <-> whole rows [nz][ny][nhp], the form of a snapshot
+// a spectrum in its blocks <-> whole rows [nz][ny][nhp], the form of a snapshot
 cudaError_t launch_spec_rows(const GridC& g, const float2* in, float2* out, bool to_rows, cudaStream_t s);
 // p_min and series sensors of one step: masked slots (p from p_sens) and u-series points
 cudaError_t launch_series(int64_t n_slots, const float* p_sens, float* p_min, const SeriesSlot* ser, float* series,

@@ -444,14 +444,15 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
         int chunk, line, l;
         place(q, chunk, line, l);
         const int mi = ISY ? l : (l == 0 ? a.load_comp[0] : (l == 1 ? a.load_comp[1] : a.load_comp[2]));
-        const CUtensorMap* map = mi == 0 ? &a.map[0] : (mi == 1 ? &a.map[1] : &a.map[2]);
         float2* dst = smem + (q % NBUF) * Line::BUF;
         uint64_t* b = &bar[q % (2 * NBUF)];
         fence_proxy_async_smem();
         mbar_arrive_expect_tx(b, Sh::STAGE * (uint32_t)sizeof(float2) + g.wait_fault_tx);
+        int w;
+        const CUtensorMap* map = tile_map<true>(a, mi, (chunk * CX) >> g.lb, w);
 #pragma unroll
         for (int k = 0; k < Sh::NBOX; ++k) {
-            const int x = (chunk * CX) & ((1 << g.lb) - 1), w = (chunk * CX) >> g.lb;
+            const int x = (chunk * CX) & ((1 << g.lb) - 1);
             if (ISY) tma_load_4d(dst + k * Sh::BOX * CX, map, x, k * Sh::BOX, line, w, b);
             else tma_load_4d(dst + k * Sh::BOX * CX, map, x, line, k * Sh::BOX, w, b);
         }

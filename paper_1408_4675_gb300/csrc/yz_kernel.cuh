@@ -1,14 +1,15 @@
 #pragma once
-// Strided-axis FFT passes on the half spectra (complex64, in blocks of 16
-// columns: kwgb_internal.h).
+// Strided-axis FFT passes on the half spectra (complex64, in blocks of 2^lb
+// columns: spec_block_log2 in kwgb_internal.h).
 //
 // Work item = a tile of CX consecutive x-columns times one whole line along
 // y (y pass) or z (z pass).  The kernels are persistent: each CTA walks its
 // share of the tiles with a two-stage shared-memory ring that the TMA unit
 // fills (cp.async.bulk.tensor, box CX x 256 lines, completion on an
 // mbarrier), so the HBM reads of tile t+1 run while tile t is transformed.
-// The ragged last tile reads the padding columns of the last block (zeros) and
-// stores none of them.
+// The ragged last tile reads padding columns, which hold anything (or, where the
+// tensor map ends with the last column, zeros); columns are never mixed, and none
+// of the padding's results is stored.
 //
 // Thread (c, j) takes elements j + TL*m of column c into registers; the
 // Stockham passes exchange through the stage buffer the tile arrived in, and
@@ -88,12 +89,14 @@ struct TShape {
 };
 
 struct alignas(64) YZK {
-    CUtensorMap map[3];       // input tensor maps (box of the pass)
+    CUtensorMap map[6];       // input tensor maps (box of the pass): every block of columns of
+                              // inputs 0 to 2, then their last blocks, clipped (kernels_yz.cu)
     GridC g;
     float2* out[3];
     int ncomp;                // y pass: components (items carry the component)
     int nloads;               // z pass: loads per item
     int load_comp[3];         // z pass: component of each load
+    int clip;                 // the block that is read through its clipped map, or -1
     int short_kappa;          // (c_ref k dt / 2)^2 <= 2 at every grid point: the short series of sinc_sq serves all
     int* flag;
 };
@@ -127,6 +130,16 @@ __device__ __forceinline__ float sinc_sq(float x2) {
     p = fmaf(p, x2, 1.0f / 120.0f);                   //  1/5!
     p = fmaf(p, x2, -1.0f / 6.0f);                    // -1/3!
     return fmaf(p, x2, 1.0f);
+}
+
+// The map of input i that holds block blk of the columns; w: the block's coordinate in it.
+// (CLIP off: the float32 passes of lines below 64 points, whose z gradient the second map
+// costs registers and a CTA per SM, 32 x 256 x 128 9.5 -> 10.5 us.)
+template <bool CLIP>
+__device__ __forceinline__ const CUtensorMap* tile_map(const YZK& a, int i, int blk, int& w) {
+    const bool last = CLIP && blk == a.clip;
+    w = last ? 0 : blk;
+    return a.map + (last ? i + 3 : i);
 }
 
 // a.out[i] for a run-time i without copying the parameter array to local memory
@@ -247,14 +260,15 @@ yz_kernel(const __grid_constant__ YZK a) {
         const int chunk = item % nchunk;
         const int line = (item / nchunk) % lines;
         const int mi = ISY ? item / (nchunk * lines) : (l == 0 ? a.load_comp[0] : (l == 1 ? a.load_comp[1] : a.load_comp[2]));
-        const CUtensorMap* map = mi == 0 ? &a.map[0] : (mi == 1 ? &a.map[1] : &a.map[2]);
         float2* dst = smem + (q % NST) * STAGE;
         uint64_t* b = &bar[q % NST];
         fence_proxy_async_smem();
         mbar_arrive_expect_tx(b, STAGE * (uint32_t)sizeof(float2) + g.wait_fault_tx);
+        int w;
+        const CUtensorMap* map = tile_map<MIXED != 0>(a, mi, (chunk * CX) >> g.lb, w);
 #pragma unroll
         for (int k = 0; k < Sh::NBOX; ++k) {
-            const int x = (chunk * CX) & ((1 << g.lb) - 1), w = (chunk * CX) >> g.lb;
+            const int x = (chunk * CX) & ((1 << g.lb) - 1);
             if (ISY) tma_load_4d(dst + k * Sh::BOX * CX, map, x, k * Sh::BOX, line, w, b);
             else tma_load_4d(dst + k * Sh::BOX * CX, map, x, line, k * Sh::BOX, w, b);
         }
