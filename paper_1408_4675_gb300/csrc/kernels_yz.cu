@@ -31,6 +31,8 @@ static EncodeTiledFn encode_fn() {
 // sectors bring their 128-byte lines), at 1024 x 1024 x 128 896 and 730.  Steps: 1024 x 1024 x 128
 // 9.06 -> 8.62 ms, 512^3 7.54 -> 7.45, 512 x 1024 x 8 0.81 -> 0.72.  Smaller spectra stay in L2, where the
 // padding costs nothing and the clipped map does (512 x 512 x 16, 34 MB, 455 -> 469 us).
+// Rows of 8 reals (5 columns of 16, next to one another) keep the promotion: it brings the rows
+// that the next tiles take (step of 1024 x 1024 x 8 1.64 -> 1.61 ms; rows of 16 reals lose 2 %).
 static bool clips_last_block(const GridC& g) { return spec_elems(g) * sizeof(float2) >= (size_t)64 << 20; }
 
 // map[0]: every block at its full width; map[1]: the last one up to the last column
@@ -49,7 +51,7 @@ static int encode_box(const GridC& g, float2* ptr, CUtensorMap (&map)[2]) {
         const cuuint64_t dims[4] = {last ? g.nh - full * w : w, (cuuint64_t)g.ny, (cuuint64_t)g.nz, last ? 1 : full + 1};
         const CUresult r = fn(&map[last], CU_TENSOR_MAP_DATA_TYPE_INT64, 4, ptr + (last ? full * spec_block(g) : 0), dims,
                               strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                              last ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              last && g.nh > 8 ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return -2;
     }

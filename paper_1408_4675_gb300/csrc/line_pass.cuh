@@ -21,7 +21,7 @@
 // take tiles in turn out of a ring of half as many buffers more, so that loads
 // are always under way while every group computes.  A CTA's tiles are
 // consecutive ones, so that the 64- or 128-byte rows in its ring are neighbours
-// in memory (tiles dealt out one by one: y 1024^3 4.96 -> 7.9 ms, z_div 512^3 0.74 ->
+// in memory (all tiles dealt out one by one: y 1024^3 4.96 -> 7.9 ms, z_div 512^3 0.74 ->
 // 0.84 ms).  The tables come from shared memory: beside the ring the L1 cache
 // is too small for them (z_abs 512^3 0.71 ms).
 #include "pair_fft.cuh"
@@ -402,9 +402,14 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
     const int nt = nchunk * lines;                            // tiles of one component
     constexpr int PER = SUM ? 3 : 1;                          // loads per unit of work
     const int units = nt * (ISY ? a.ncomp : (STASH ? 1 : a.nloads));
-    // consecutive units, so that the tiles in a CTA's ring are neighbours in memory
-    const int u0 = (int)((int64_t)units * blockIdx.x / gridDim.x);
-    const int my = (int)((int64_t)units * (blockIdx.x + 1) / gridDim.x) - u0;
+    // Consecutive units, so that the tiles in a CTA's ring are neighbours in memory; with one
+    // tile to a line (rows of 8 or 16 reals) dealt out one by one, so that the tiles of all
+    // CTAs are (steps of 1024 x 1024 x 8 1.68 -> 1.64 ms, 512 x 512 x 8 308 -> 304 us).
+    const bool one = nchunk == 1;
+    const int u0 = one ? (int)blockIdx.x : (int)((int64_t)units * blockIdx.x / gridDim.x);
+    const int my = one ? (units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1
+                       : (int)((int64_t)units * (blockIdx.x + 1) / gridDim.x) - u0;
+    const int us = one ? (int)gridDim.x : 1;
     const int Q = my * PER;
     auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(THREADS) : "memory"); };
 
@@ -431,7 +436,7 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
     }
 
     auto place = [&](int q, int& chunk, int& line, int& l) {
-        int u = u0 + q / PER;
+        int u = u0 + q / PER * us;
         if (SUM) l = q % PER;
         else {
             l = u / nt;

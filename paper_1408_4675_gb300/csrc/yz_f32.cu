@@ -17,6 +17,12 @@ namespace kwgb {
 
 template <int L, int OP>
 static cudaError_t launch_f32(const YZK& a, int items, cudaStream_t s) {
+    // y lines of 1024 points of 8-real rows, in spectra beyond L2: HBM bounds the pass and 3 of
+    // a tile's 8 columns are idle, so one-exchange transforms save nothing, and the one-column kernel
+    // is faster (step of 1024 x 1024 x 8 1.61 -> 1.58 ms; in L2, 256 x 1024 x 8, 317 -> 348 us)
+    if constexpr (L == 10 && OP < 2) {
+        if (a.clip == 0 && a.g.nh <= 8) return launch_t<L, OP, 0>(a, items, s);
+    }
     if constexpr (L >= 6) return launch_line<L, OP>(a, s);
     else return launch_t<L, OP, 0>(a, items, s);
 }

@@ -133,7 +133,7 @@ __device__ __forceinline__ float sinc_sq(float x2) {
 }
 
 // The map of input i that holds block blk of the columns; w: the block's coordinate in it.
-// (CLIP off: the float32 passes of lines below 64 points, whose z gradient the second map
+// (CLIP off: the passes of lines below 64 points, whose float32 z gradient the second map
 // costs registers and a CTA per SM, 32 x 256 x 128 9.5 -> 10.5 us.)
 template <bool CLIP>
 __device__ __forceinline__ const CUtensorMap* tile_map(const YZK& a, int i, int blk, int& w) {
@@ -265,7 +265,7 @@ yz_kernel(const __grid_constant__ YZK a) {
         fence_proxy_async_smem();
         mbar_arrive_expect_tx(b, STAGE * (uint32_t)sizeof(float2) + g.wait_fault_tx);
         int w;
-        const CUtensorMap* map = tile_map<MIXED != 0>(a, mi, (chunk * CX) >> g.lb, w);
+        const CUtensorMap* map = tile_map<(LOGN >= 6)>(a, mi, (chunk * CX) >> g.lb, w);
 #pragma unroll
         for (int k = 0; k < Sh::NBOX; ++k) {
             const int x = (chunk * CX) & ((1 << g.lb) - 1);
