@@ -374,6 +374,9 @@ __device__ __forceinline__ void stash_get(uint32_t taddr, float2 (&re)[H], float
 // NBUF and is handled by group t mod GR (DIV_SUM: the three loads of a tile by
 // one group); the group that has read load t's buffer for the last time issues
 // load t + NBUF into it.
+// A group whose wait runs out takes no more tiles.  Groups that it would have fed run
+// out in turn, and before the CTA exits every load that was issued and not waited for gets one more
+// bounded wait: the TMA must not write into shared memory that is no longer the CTA's.
 template <int LOGN, int OP>
 __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZK a) {
     constexpr bool ISY = OP < 2;
@@ -386,7 +389,7 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
     constexpr bool STASH = GRAD || SUM;
     constexpr bool BWD = OP == OP_Z_GRAD_BWD || OP == OP_Z_DIV || SUM;    // e^{-ikd/2}: the real part of the operator negated
     extern __shared__ __align__(128) float2 smem[];
-    __shared__ int abort_flag[GR];
+    __shared__ int stop[GR];                                  // the load at which a group gave up, or -1
     __shared__ uint32_t tslot;
     // the tables that every thread reads for every value: from shared memory, since
     // the ring leaves the L1 cache too small to keep them
@@ -419,7 +422,7 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
         for (int i = 0; i < 2 * NBUF; ++i) mbar_init(&bar[i], 1);
         fence_mbar_init();
     }
-    if (tid == 0) abort_flag[grp] = 0;
+    if (tid == 0) stop[grp] = -1;
     for (int i = threadIdx.x; i < (ISY ? Line::NTW : Line::NTW2); i += 512) tw[i] = __ldg(g.t.tw + Line::TW0 + i);
     if (!ISY)
         for (int i = threadIdx.x; i < (1 << LOGN); i += 512) {
@@ -465,6 +468,7 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
     after_previous();
     if (threadIdx.x == 0)
         for (int q = 0; q < NBUF && q < Q; ++q) issue(q);
+    bool gave_up = false;
     for (int i = grp; i < my; i += GR) {
     for (int q = i * PER; q < (i + 1) * PER; ++q) {
         int chunk, line, l;
@@ -493,7 +497,7 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
         // previous phase is known to be over.  Load q has barrier q mod 2 NBUF: the load before
         // on it (q - 2 NBUF) was this group's own, since GR divides 2 NBUF.
         const bool ok = mbar_wait_bounded(&bar[q % (2 * NBUF)], (q / (2 * NBUF)) & 1, a.flag);
-        if (!ok) abort_flag[grp] = 1;
+        if (!ok) stop[grp] = q;
         float2 re[H], im[H];
         // the buffer is free for its next load once every thread of the group has read it
         auto next = [&]() {
@@ -501,10 +505,9 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
             if (tid == 0 && q + NBUF < Q) issue(q + NBUF);
         };
         Line::template fwd<OP == OP_Y_INV>(re, im, buf, c, j, tw, sync);
-        if (abort_flag[grp]) {                        // set before fwd's barriers, so the same for the whole group
-            // no more tiles for this group; a load of its own still under way is waited for (bounded)
-            if (tid == 0 && q + GR < Q && q + GR < NBUF) mbar_wait_bounded(&bar[q + GR], 0, a.flag);
-            i = my;
+        if (stop[grp] >= 0) {                         // set before fwd's barriers, so the same for the whole group
+            gave_up = true;
+            i = my;                                   // no more tiles for this group
             break;
         }
         if constexpr (ISY) {
@@ -607,6 +610,17 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
             });
         }
     }
+    }
+    if (__syncthreads_or(gave_up) && threadIdx.x < 4 * GR) {  // every group has finished or given up
+        // A load is issued when the one NBUF before it has been released, and a group releases its loads
+        // in order, up to stop[].  The loads of a group beyond that which are issued are among its next
+        // three (the groups feed each other in pairs): one to a lane, so that the waits run side by side.
+        const int gr = threadIdx.x / 4;
+        const int n = stop[gr] / (PER * GR) * PER + stop[gr] % PER + threadIdx.x % 4;   // the group's n-th load
+        const int q = (n / PER * GR + gr) * PER + n % PER;
+        const int feeder = (q - NBUF) / PER % GR;
+        if (stop[gr] >= 0 && q < Q && (q < NBUF || stop[feeder] < 0 || q - NBUF < stop[feeder]))
+            mbar_wait_bounded(&bar[q % (2 * NBUF)], (q / (2 * NBUF)) & 1, a.flag);
     }
     if (STASH) {
         tc5_fence_before();
