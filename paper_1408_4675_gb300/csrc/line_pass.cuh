@@ -635,12 +635,15 @@ inline cudaError_t launch_line(const YZK& a, cudaStream_t s) {
     using Ls = LShape<LOGN, (OP < 2)>;
     constexpr bool stash = OP == OP_Z_GRAD_FWD || OP == OP_Z_GRAD_BWD || OP == OP_Z_DIV_SUM;
     auto k = line_kernel<LOGN, OP>;
-    static bool ready = false;
-    if (!ready) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Ls::SMEM);
-        if (e != cudaSuccess) return e;
-        ready = true;
-    }
+    static PerDevice ready;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    ready.get(dev, [&] {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Ls::SMEM);
+        return e == cudaSuccess ? 1 : 0;
+    });
+    if (e != cudaSuccess) return e;
     const int nchunk = (a.g.nh + Ls::Sh::CX - 1) / Ls::Sh::CX;
     const int lines = OP < 2 ? a.g.nz : a.g.ny;
     const int units = nchunk * lines * (OP < 2 ? a.ncomp : (stash ? 1 : a.nloads));

@@ -29,6 +29,7 @@
 #include "fft_tc5.cuh"
 #include "kwgb_internal.h"
 #include "launch.cuh"
+#include "per_device.h"
 #include "tma.cuh"
 
 namespace kwgb {
@@ -451,34 +452,36 @@ template <int LOGN, int OP, int MIXED>
 inline cudaError_t launch_t(const YZK& a, int items, cudaStream_t s) {
     using Sh = TShape<LOGN, (OP < 2), MIXED>;
     auto k = yz_kernel<LOGN, OP, MIXED>;
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::smem(MIXED));
-        if (e != cudaSuccess) return e;
-        if (Sh::TC5) {
+    static PerDevice resident;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const int per_sm = resident.get(dev, [&] {
+        int n = 0;
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::smem(MIXED));
+        if (e == cudaSuccess && Sh::TC5)
             e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-            if (e != cudaSuccess) return e;
-        }
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Sh::THREADS, Sh::smem(MIXED));
-        if (e != cudaSuccess) return e;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, Sh::THREADS, Sh::smem(MIXED));
+        if (e != cudaSuccess) return 0;
         if (Sh::TC5) {
             // residency from the kernel's registers and shared memory (the query
             // has returned less than the hardware holds for the tensor-core form);
             // each resident CTA holds TC5_TMEM of the 512 tensor-memory columns
             cudaFuncAttributes fa;
-            int dev = 0, smem_sm = 0, regs_sm = 0;
-            if (cudaFuncGetAttributes(&fa, k) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
+            int smem_sm = 0, regs_sm = 0;
+            if (cudaFuncGetAttributes(&fa, k) == cudaSuccess &&
                 cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess &&
                 cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) == cudaSuccess) {
                 const int per_block = Sh::smem(MIXED) + (int)fa.sharedSizeBytes + 1024;
                 const int regs = ((fa.numRegs + 7) / 8) * 8 * Sh::THREADS;
                 int m = std::min(smem_sm / per_block, regs_sm / std::max(regs, 1));
                 m = std::min(m, 512 / Sh::TC5_TMEM);
-                per_sm = std::max(per_sm, m);
+                n = std::max(n, m);
             }
         }
-        if (per_sm < 1) per_sm = 1;
-    }
+        return std::max(n, 1);
+    });
+    if (e != cudaSuccess) return e;
     int grid = per_sm * a.g.num_sms;
     if (grid > items) grid = items;
     if (grid < 1) return cudaSuccess;
