@@ -393,6 +393,14 @@ int kwgb_status(kwgb_sim* sim);
  * Errors: ARG. */
 int kwgb_debug_wait_fault(kwgb_sim* sim, int on);
 
+/* Test hook of the same path: the next n captures of steps into a CUDA graph
+ * break off after their first step (on the host; nothing is launched).  The
+ * library then launches directly, or one step at a time where only the capture of
+ * several steps failed, and does not try that capture again.  Returns the
+ * failures that an earlier call asked for and that have not happened.  Errors:
+ * ARG. */
+int kwgb_debug_capture_fault(kwgb_sim* sim, int n);
+
 /* Device bytes held by the simulation. */
 int64_t kwgb_device_bytes(const kwgb_sim* sim);
 

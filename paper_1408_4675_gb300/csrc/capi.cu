@@ -132,6 +132,8 @@ struct kwgb_sim {
     cudaStream_t cap = nullptr;         // stream the step is captured on
     int64_t glaunches = 0;              // kernels in a captured step
     bool graph_off = false;             // capture not possible: launch directly
+    bool graph_n_off = false;           // of kGraphSteps steps not possible: one step at a time
+    int capture_faults = 0;             // test hook: captures still to fail
     bool warmed = false;                // a step has run directly (one-time set-up done)
     // per-launch event timing (kwgb_step_profiled)
     bool prof = false;
@@ -594,15 +596,20 @@ static cudaGraphExec_t capture_steps(kwgb_sim* sim, int count) {
     const std::string err = sim->err;
     sim->prof = false;
     int e = KWGB_OK;
-    for (int i = 0; i < count && e == KWGB_OK; ++i) e = launch_step(sim, sim->cap);
+    for (int i = 0; i < count && e == KWGB_OK; ++i) {
+        e = launch_step(sim, sim->cap);
+        if (sim->capture_faults > 0) e = KWGB_ERR_CUDA;
+    }
+    if (sim->capture_faults > 0) sim->capture_faults--;
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(sim->cap, &graph);
     sim->prof = prof;
-    sim->glaunches = (sim->launches - l0) / count;
+    const int64_t per_step = (sim->launches - l0) / count;   // (if every step was captured)
     sim->launches = l0;
     sim->err = err;
     cudaGraphExec_t exec = nullptr;
     if (e != KWGB_OK || ce != cudaSuccess || !graph || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) exec = nullptr;
+    if (exec) sim->glaunches = per_step;
     if (graph) cudaGraphDestroy(graph);
     cudaGetLastError();
     return exec;
@@ -613,6 +620,7 @@ static void drop_graphs(kwgb_sim* sim) {
     if (sim->gexec) cudaGraphExecDestroy(sim->gexec);
     if (sim->gexec_n) cudaGraphExecDestroy(sim->gexec_n);
     sim->gexec = sim->gexec_n = nullptr;
+    sim->graph_n_off = false;
 }
 
 // n steps on stream s: the captured graphs when there are any, else direct launches.
@@ -634,7 +642,10 @@ static int run_steps(kwgb_sim* sim, int64_t n, cudaStream_t s) {
             n--;
             continue;
         }
-        if (n >= 8 * kGraphSteps && !sim->gexec_n) sim->gexec_n = capture_steps(sim, kGraphSteps);
+        if (n >= 8 * kGraphSteps && !sim->gexec_n && !sim->graph_n_off) {
+            sim->gexec_n = capture_steps(sim, kGraphSteps);
+            sim->graph_n_off = sim->gexec_n == nullptr;
+        }
         const bool many = n >= kGraphSteps && sim->gexec_n;
         CK(cudaGraphLaunch(many ? sim->gexec_n : sim->gexec, s));
         const int k = many ? kGraphSteps : 1;
@@ -1629,6 +1640,13 @@ extern "C" int kwgb_debug_wait_fault(kwgb_sim* sim, int on) {
 }
 
 extern "C" int64_t kwgb_device_bytes(const kwgb_sim* sim) { return sim ? sim->bytes : 0; }
+
+extern "C" int kwgb_debug_capture_fault(kwgb_sim* sim, int n) {
+    if (!sim || n < 0) return KWGB_ERR_ARG;
+    const int left = sim->capture_faults;
+    sim->capture_faults = n;
+    return left;
+}
 
 extern "C" const char* kwgb_last_error(const kwgb_sim* sim) {
     return sim ? sim->err.c_str() : g_create_error.c_str();

@@ -101,6 +101,8 @@ def load():
     L.kwgb_load_state.restype = ctypes.c_int
     L.kwgb_debug_wait_fault.argtypes = [vp, ctypes.c_int]
     L.kwgb_debug_wait_fault.restype = ctypes.c_int
+    L.kwgb_debug_capture_fault.argtypes = [vp, ctypes.c_int]
+    L.kwgb_debug_capture_fault.restype = ctypes.c_int
     L.kwgb_gradient_static.argtypes = [ctypes.POINTER(GridDesc), ctypes.c_int, vp, vp, vp, vp, vp,
                                        ctypes.c_char_p, ctypes.c_size_t]
     L.kwgb_gradient_static.restype = ctypes.c_int
