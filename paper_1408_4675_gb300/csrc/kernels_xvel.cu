@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_vel_ke
     const GridC& g = K.g;
     const int r = threadIdx.x / TL, j = threadIdx.x % TL;
     const int nrows = g.ny * g.nz;
-        const int row = (ONE ? blockIdx.x / 3 : blockIdx.x) * Sh::RPB + r;
+    const int row = (ONE ? blockIdx.x / 3 : blockIdx.x) * Sh::RPB + r;
     const bool valid = row < nrows;
     const int rr = valid ? row : 0;
     const int y = rr % g.ny, z = rr / g.ny;
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(XShape<LOGM>::XT, XShape<LOGM>::MINB) x_vel_ke
                 }
             }
         }
-        if (MODE == XV_STEP) row_r2c<LOGM, (LOGM >= 9)>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(pick3w(K.a.U, xi), rr), g);
+        if (MODE == XV_STEP) row_r2c<LOGM>(v, S, j, valid, g.t.tw, spec_row<Sh::M>(pick3w(K.a.U, xi), rr), g);
     };
     if (ONE) component(blockIdx.x % 3);
     else {

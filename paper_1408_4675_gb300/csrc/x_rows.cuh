@@ -92,21 +92,35 @@ struct XShape {
     }
 };
 
-// exp(DIR 2 pi i k / (2M)) for k = j + TL*m.  ONE: one table load per thread (w0 =
-// the value at k = j) times the compile-time root exp(DIR i pi m / E) (TL / M = 1 / E),
-// instead of E loads.  Which is faster depends on the kernel (ms at 512^3, ONE / table: x_dens
-// 1.273 / 1.307, x_eos 0.788 / 0.806, x_vel 1.405 / 1.340; rows of 1024 reals: ONE everywhere).
-template <bool ONE, int DIR, int M, int E>
+// exp(DIR 2 pi i k / (2M)) for k = j + TL*m, by FORM:
+//   TW_TABLE  the table entry of k
+//   TW_HALF   the entries of the first half of the m, the others those times DIR i (TL / M = 1 / E): as
+//             accurate, half the loads
+//   TW_ONE    one load per thread (w0 = the value at k = j) times the compile-time root
+//             exp(DIR i pi m / E); the root's rounding and the product's come on top
+enum { TW_TABLE, TW_HALF, TW_ONE };
+template <int FORM, int DIR, int M, int E>
 __device__ __forceinline__ float2 row_tw(const float2* __restrict__ tw, float2 w0, int k, int m) {
     static_assert(E <= 8 && 8 % E == 0, "roots of 16");
-    if constexpr (ONE) return rot16<DIR>(w0, m * (8 / E));
-    else return row_twiddle<DIR, M>(tw, k);
+    if constexpr (FORM == TW_ONE) return rot16<DIR>(w0, m * (8 / E));
+    if constexpr (FORM == TW_HALF) {
+        if (m < E / 2) return row_twiddle<DIR, M>(tw, k);
+        const float2 w = row_twiddle<DIR, M>(tw, k - M / 2);
+        return DIR > 0 ? make_float2(-w.y, w.x) : make_float2(w.y, -w.x);
+    }
+    return row_twiddle<DIR, M>(tw, k);
 }
-template <bool ONE, int DIR, int M>
+template <int FORM, int DIR, int M>
 __device__ __forceinline__ float2 row_tw0(const float2* __restrict__ tw, int j) {
-    if constexpr (ONE) return row_twiddle<DIR, M>(tw, j);
+    if constexpr (FORM == TW_ONE) return row_twiddle<DIR, M>(tw, j);
     else return make_float2(0.f, 0.f);
 }
+// Rows of 1024 reals: one load; 512: half the loads (step of 512^3 7.36 ms, with the table 7.46, with one
+// load 7.37); shorter rows: the table (256^3 0.963 ms, half the loads 0.976, one load 0.960).  One load
+// below 1024 reals cost accuracy: error of gradients of 64 x 64 x 512 against float64 4.08e-7 -> 4.11e-7, of a
+// step's p_max at 256^3 3.09e-7 -> 3.20e-7.
+template <int M>
+__host__ __device__ constexpr int tw_form() { return M >= 512 ? TW_ONE : (M >= 256 ? TW_HALF : TW_TABLE); }
 
 // Unnormalised C2R of one row: spec[0..M] (Hermitian half spectrum) ->
 // z[m] = (x[2n], x[2n+1]) with n = j + TL*m and
@@ -128,13 +142,13 @@ __device__ __forceinline__ void row_c2r_lds(const float2* __restrict__ spec, con
     for (int m = 0; m < E; ++m) S.at(j + TL * m) = t[m];
     if (j == 0) S.at(M) = nyq;
     S.sync();
-    const float2 w0 = row_tw0<(M >= 512), +1, M>(tw, j);
+    const float2 w0 = row_tw0<TW_ONE, +1, M>(tw, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int k = j + TL * m;
         const float2 xk = S.at(k), xm = cconj(S.at(M - k));
         const float2 a = cadd(xk, xm);
-        const float2 b = cmul(csub(xk, xm), row_tw<(M >= 512), +1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
+        const float2 b = cmul(csub(xk, xm), row_tw<TW_ONE, +1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
         z[m] = make_float2(a.x - b.y, a.y + b.x);                                // a + i b
     }
     line_fft<LOGM, E, +1>(z, j, S, tw);
@@ -163,24 +177,23 @@ __device__ __forceinline__ void row_c2r_shfl(const float2* __restrict__ spec, co
 #pragma unroll
     for (int m = 0; m < E; ++m) t[m] = valid ? __ldcs(spec_at<M>(spec, g, j + TL * m)) : make_float2(0.f, 0.f);
     if (valid && j == 0) nyq = __ldcs(spec_at<M>(spec, g, M));
-    const float2 w0 = row_tw0<(M >= 512), +1, M>(tw, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int k = j + TL * m;
         const float2 xm = cconj(mirrored<TL, E>(t, nyq, j, m));
         const float2 a = cadd(t[m], xm);
-        const float2 b = cmul(csub(t[m], xm), row_tw<(M >= 512), +1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
+        const float2 b = cmul(csub(t[m], xm), row_twiddle<+1, M>(tw, k));   // exp(+2 pi i k / nx)
         z[m] = make_float2(a.x - b.y, a.y + b.x);                                  // a + i b
     }
     line_fft<LOGM, E, +1>(z, j, S, tw);
 }
-template <int LOGM, bool ONE>
+template <int LOGM, int FORM>
 __device__ __forceinline__ void row_r2c_shfl(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
                                              bool valid, const float2* __restrict__ tw, float2* __restrict__ spec, const GridC& g) {
     using Sh = XShape<LOGM>;
     constexpr int M = Sh::M, E = Sh::E, TL = Sh::TL;
     line_fft<LOGM, E, -1>(z, j, S, tw);
-    const float2 w0 = row_tw0<ONE, -1, M>(tw, j);
+    const float2 w0 = row_tw0<FORM, -1, M>(tw, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int k = j + TL * m;
@@ -188,7 +201,7 @@ __device__ __forceinline__ void row_r2c_shfl(float2 (&z)[XShape<LOGM>::E], typen
         const float2 s = cadd(z[m], zm), d = csub(z[m], zm);
         const float2 xe = make_float2(0.5f * s.x, 0.5f * s.y);
         const float2 xo = make_float2(0.5f * d.y, -0.5f * d.x);              // d / (2i)
-        const float2 x = cadd(xe, cmul(xo, row_tw<ONE, -1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
+        const float2 x = cadd(xe, cmul(xo, row_tw<FORM, -1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
         if (valid) {
             __stcs(spec_at<M>(spec, g, k), x);
             if (k == 0) __stcs(spec_at<M>(spec, g, M), csub(xe, xo));
@@ -245,20 +258,20 @@ __device__ __forceinline__ void row_c2r_staged(const float2* srow, typename XSha
                                                float2 (&z)[XShape<LOGM>::E]) {
     using Sh = XShape<LOGM>;
     constexpr int M = Sh::M, E = Sh::E, TL = Sh::TL;
-    const float2 w0 = row_tw0<(M >= 128), +1, M>(tw, j);
+    const float2 w0 = row_tw0<tw_form<M>(), +1, M>(tw, j);
 #pragma unroll
     for (int m = 0; m < E; ++m) {
         const int k = j + TL * m;
         const float2 xk = srow[k], xm = cconj(srow[M - k]);
         const float2 a = cadd(xk, xm);
-        const float2 b = cmul(csub(xk, xm), row_tw<(M >= 128), +1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
+        const float2 b = cmul(csub(xk, xm), row_tw<tw_form<M>(), +1, M, E>(tw, w0, k, m));   // exp(+2 pi i k / nx)
         z[m] = make_float2(a.x - b.y, a.y + b.x);                                // a + i b
     }
     S.sync();                                        // previous users of the work row are done
     line_fft<LOGM, E, +1>(z, j, S, tw);
 }
 
-template <int LOGM, bool ONE>
+template <int LOGM, int FORM>
 __device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
                                         bool valid, const float2* __restrict__ tw,
                                         float2* __restrict__ spec, const GridC& g) {
@@ -270,7 +283,7 @@ __device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typen
     for (int m = 0; m < E; ++m) S.at(j + TL * m) = z[m];
     S.sync();
     if (valid) {
-        const float2 w0 = row_tw0<ONE, -1, M>(tw, j);
+        const float2 w0 = row_tw0<FORM, -1, M>(tw, j);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int k = j + TL * m;
@@ -278,7 +291,7 @@ __device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typen
             const float2 s = cadd(zk, zm), d = csub(zk, zm);
             const float2 xe = make_float2(0.5f * s.x, 0.5f * s.y);
             const float2 xo = make_float2(0.5f * d.y, -0.5f * d.x);              // d / (2i)
-            const float2 x = cadd(xe, cmul(xo, row_tw<ONE, -1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
+            const float2 x = cadd(xe, cmul(xo, row_tw<FORM, -1, M, E>(tw, w0, k, m)));   // exp(-2 pi i k / nx)
             __stcs(spec_at<M>(spec, g, k), x);
             if (k == 0) __stcs(spec_at<M>(spec, g, M), csub(xe, xo));
         }
@@ -286,12 +299,12 @@ __device__ __forceinline__ void row_r2c_smem(float2 (&z)[XShape<LOGM>::E], typen
 }
 
 // Unnormalised R2C of one row: z[m] = (x[2n], x[2n+1]) -> spec[0..M].
-template <int LOGM, bool ONE = (LOGM >= 7)>
+template <int LOGM, int FORM = tw_form<(1 << LOGM)>()>
 __device__ __forceinline__ void row_r2c(float2 (&z)[XShape<LOGM>::E], typename XShape<LOGM>::Smem& S, int j,
                                         bool valid, const float2* __restrict__ tw,
                                         float2* __restrict__ spec, const GridC& g) {
-    if constexpr (XShape<LOGM>::SHFL) row_r2c_shfl<LOGM, ONE>(z, S, j, valid, tw, spec, g);
-    else row_r2c_smem<LOGM, ONE>(z, S, j, valid, tw, spec, g);
+    if constexpr (XShape<LOGM>::SHFL) row_r2c_shfl<LOGM, FORM>(z, S, j, valid, tw, spec, g);
+    else row_r2c_smem<LOGM, FORM>(z, S, j, valid, tw, spec, g);
 }
 
 template <int LOGM>
