@@ -127,7 +127,8 @@ __device__ __forceinline__ float2 rot32(float2 d, int m) {
     if (m == 0) return d;
     if (m == 8) return make_float2(d.y, -d.x);
     const float c = cos32(m), s = -sin32(m);
-    return make_float2(fmaf(d.x, c, -d.y * s), fmaf(d.x, s, d.y * c));
+    if (m > 4 && m < 12) return make_float2(fmaf(-d.y, s, d.x * c), fmaf(d.x, s, d.y * c));   // (the order: cmul2_flat)
+    return make_float2(fmaf(d.x, c, -d.y * s), fmaf(d.y, c, d.x * s));
 }
 
 // 32 elements of one column, N = 32 TL.  Forward: 32-point butterflies over the

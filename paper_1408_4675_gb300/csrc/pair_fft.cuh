@@ -40,14 +40,25 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 __device__ __forceinline__ float2 dup2(float s) { return make_float2(s, s); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
-// (re, im) *= (c + i s), packed: re' = re c - im s, im' = im c + re s.
+// (re, im) *= (c + i s), packed: re' = re c - im s, im' = im c + re s.  Of each sum's two products one
+// is rounded by itself, the other within the fma; better the smaller one, so constant factors nearer
+// to 1 than to i take cmul2_flat.  (For table twiddles it makes no difference that can be measured, and the
+// other order costs the 512-point gradient pass registers: 1.985 -> 2.047 ms at 512^3.)
 __device__ __forceinline__ void cmul2(float2& re, float2& im, float2 c, float2 s) {
     const float2 r = fma2(im, neg2(s), mul2(re, c));
     im = fma2(re, s, mul2(im, c));
     re = r;
 }
+__device__ __forceinline__ void cmul2_flat(float2& re, float2& im, float2 c, float2 s) {
+    const float2 r = fma2(re, c, mul2(im, neg2(s)));
+    im = fma2(im, c, mul2(re, s));
+    re = r;
+}
 
-// (re, im) *= exp(-2 pi i m / 16) for a compile-time m in [0, 8).
+// exp(-2 pi i m / 16) is nearer to +-i than to +-1
+__host__ __device__ constexpr bool steep16(int m) { return (m & 7) > 2 && (m & 7) < 6; }
+
+// (re, im) *= exp(-2 pi i m / 16) for a compile-time m in [0, 16), m != 8, 12.
 __device__ __forceinline__ void rot2(float2& re, float2& im, int m) {
     if (m == 0) return;
     if (m == 4) {                                     // * -i
@@ -56,7 +67,8 @@ __device__ __forceinline__ void rot2(float2& re, float2& im, int m) {
         re = r;
         return;
     }
-    cmul2(re, im, dup2(cos16(m)), dup2(-sin16(m)));
+    if (steep16(m)) cmul2(re, im, dup2(cos16(m)), dup2(-sin16(m)));
+    else cmul2_flat(re, im, dup2(cos16(m)), dup2(-sin16(m)));
 }
 
 // Forward DFT of four values at a, b, c, d, in place (output k in the k-th).
@@ -75,16 +87,13 @@ __device__ __forceinline__ void dft4_pair(float2* re, float2* im, int a, int b, 
 
 // Sixteen values as 4 x 4: 8 of them are rotated (and rounded) once, against 10 rotations in the
 // radix-2 form; with those a line of 512 points was less accurate than three radix-8 passes
-// (1.08e-7 relative error against 1.02e-7; now 1.05e-7).
+// (1.08e-7 relative error against 1.02e-7; now 1.05e-7, and 1.04e-7 with the order of cmul2_flat).
 __device__ __forceinline__ void dft16_pair(float2* re, float2* im) {
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
         dft4_pair(re, im, n, n + 4, n + 8, n + 12);
 #pragma unroll
-        for (int k = 1; k < 4; ++k) {
-            if (n * k <= 7) rot2(re[n + 4 * k], im[n + 4 * k], n * k);
-            else cmul2(re[n + 4 * k], im[n + 4 * k], dup2(cos16(n * k)), dup2(-sin16(n * k)));
-        }
+        for (int k = 1; k < 4; ++k) rot2(re[n + 4 * k], im[n + 4 * k], n * k);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) dft4_pair(re, im, 4 * k, 4 * k + 1, 4 * k + 2, 4 * k + 3);   // output k + 4 q at 4 k + q
