@@ -2,7 +2,8 @@
 // the host in float64), the sparse source/sensor structures, and the launch
 // sequence of one time step.
 //
-// Device memory of a simulation (F = nx*ny*nz floats, S = nz*ny*nhp complex):
+// Device memory of a simulation (F = nx*ny*nz floats, S = spec_elems complex: nz*ny times nx/2 + 1
+// columns in whole blocks of 16 or 32, kwgb_internal.h):
 //   u_x, u_y, u_z, rho_x, rho_y, rho_z        6 F   state
 //   c0, rho0, B/A, alpha0                     <= 4 F (scalars take no memory)
 //   P (x-transformed p^n), T1, T2, T3         4 S   spectra; T1/T2 hold the
@@ -430,7 +431,7 @@ extern "C" int kwgb_set_medium(kwgb_sim* sim, const float* c0, const float* rho0
     DALLOC(sim->T1, float2, sim->spec_elems);
     DALLOC(sim->T2, float2, sim->spec_elems);
     DALLOC(sim->T3, float2, sim->spec_elems);
-    for (float2* p : {sim->P, sim->T1, sim->T2, sim->T3}) CK(cudaMemset(p, 0, sim->spec_elems * sizeof(float2)));
+    CK(cudaMemset(sim->P, 0, sim->spec_elems * sizeof(float2)));   // the others are written before they are read
     {
         int sms = 0;
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id));
