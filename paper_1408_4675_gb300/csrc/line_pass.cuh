@@ -299,8 +299,8 @@ struct LShape {
 // exp2 of the operator exponents e log2(k^2 / k_max^2), |e| < 1: the hardware function without the
 // handling of denormal results, the same as exp2f there (compared for every float k^2 / k_max^2 in [2^-40, 4)).
 // The logarithm is log2f: lg2.approx differs from it in a third of those arguments, by up to
-// a unit in the last place more, which the powers multiply (error of k^{y-2} at 256^3 2.8e-7 -> 3.6e-7;
-// z_abs would be a tenth faster, the eta operator of 256^3 117 us instead of 124).
+// a unit in the last place more, which the powers multiply (error of k^{y-2} at 256^3 2.7e-7 -> 3.5e-7;
+// z_abs would take 0.445 ms at 512^3 instead of 0.468, the eta operator of 256^3 117 us instead of 124).
 __device__ __forceinline__ float ex2_normal(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -562,6 +562,7 @@ __global__ void __launch_bounds__(512, 1) line_kernel(const __grid_constant__ YZ
             else apply(std::false_type{});
             if (GRAD) stash_put(taddr, re, im);
             if (SUM) {
+                // (the stashed values beside the live ones: up to 60 bytes of spill loads a thread, 618 for 256-point lines)
                 if (comp > 0) {
                     float2 sr[H], si[H];
                     stash_get(taddr, sr, si);

@@ -20,8 +20,8 @@
 // x = 2(j + TL*m), so every global access of a row is coalesced.  A "team"
 // is the smallest set of whole warps that holds whole rows: one warp with
 // 32/TL rows (TL <= 32), or the TL/32 warps of one row (1024-point rows:
-// E = 8, TL = 64, two warps, so that the kernels keep two CTAs per SM
-// instead of spilling 16 values per thread at one CTA).  All synchronisation
+// E = 8, TL = 64, two warps, so that the kernels keep 16 warps per SM
+// instead of spilling 16 values per thread in half as many).  All synchronisation
 // is within a team (a warp barrier, or a named barrier per team), so the
 // teams of a CTA stream their rows independently.
 #pragma once

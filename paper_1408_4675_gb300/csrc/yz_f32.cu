@@ -7,9 +7,9 @@
 // (32^3 step 44.6 -> 46.1 us).
 // Against the kernels they replaced (8 or 16 values per thread, two exchanges
 // per transform, three for 1024 points), z_div / z_abs / y of three spectra:
-//   512^3   0.991 / 0.663 / 0.565 ms -> 0.682 / 0.439 / 0.569 ms
-//   1024^3 11.12  / 6.93  / 5.0  ms -> 6.22  / 3.76  / 4.75 ms
-//   256^3   133   / 90    / 76   us -> 91    / 59    / 78   us
+//   512^3   0.991 / 0.663 / 0.565 ms -> 0.657 / 0.468 / 0.555 ms
+//   1024^3 11.12  / 6.93  / 5.0  ms -> 6.16  / 4.17  / 4.53 ms
+//   256^3   133   / 90    / 76   us -> 89    / 74    / 75   us
 // (with the spectra in blocks of columns, kwgb_internal.h).
 #include "line_pass.cuh"
 

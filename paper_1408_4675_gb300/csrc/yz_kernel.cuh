@@ -56,6 +56,9 @@ struct TileSmem {
     __device__ __forceinline__ void sync() { __syncthreads(); }
 };
 
+// The tiles of a pass.  The float32 passes of lines of 64 points and more run on line_kernel
+// (line_pass.cuh), which takes the tile width CX and the boxes from here; E, TL and THREADS then serve the
+// 1024-point y lines of 8-real rows alone (yz_f32.cu).
 // MIXED: the tensor-core forms take 8-column tiles of 256 threads for 512-point
 // y lines (64 KB per CTA: two CTAs per SM; the float32 y pass keeps 16 columns)
 template <int LOGN, bool ISY, int MIXED = 0>
